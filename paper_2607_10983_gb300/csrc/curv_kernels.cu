@@ -277,63 +277,49 @@ __global__ void k_curv_apply(Dims d, CurvCoef cf, const T* __restrict__ u, T* __
   out[i] = v;
 }
 
-// out = r - op(u) / J, with optional block partial sums of out^2
-template <typename T>
-__global__ void k_curv_residual(Dims d, CurvCoef cf, const T* __restrict__ r, const T* __restrict__ u,
-                                T* __restrict__ out, T inv_h2, int form, double* __restrict__ partials) {
-  __shared__ double sh[32];
+// out = r - op(u) / J
+__global__ void k_curv_residual(Dims d, CurvCoef cf, const float* __restrict__ r, const float* __restrict__ u,
+                                float* __restrict__ out, float inv_h2, int form) {
   const int x = blockIdx.x * BX + threadIdx.x, y = blockIdx.y * BY + threadIdx.y, z = blockIdx.z;
-  T res = T(0);
-  if (x < d.nx && y < d.ny) {
-    const Nbhd nb(d, x, y, z);
-    const FieldAt<T> U{u, &nb};
-    const CoefAt Bc{cf, &nb};
-    const long long i = nb(0, 0, 0);
-    res = r[i] - op_h2<T>(U, Bc, form) * inv_h2 / T(cf.J[i]);
-    out[i] = res;
-  }
-  if (partials) {
-    double s;
-    if constexpr (sizeof(T) == 8) s = block_sum((double)res * (double)res, sh);
-    else s = block_sum_f(res * res, sh);
-    if (is_thread0()) partials[block_linear_id()] = s;
-  }
+  if (x >= d.nx || y >= d.ny) return;
+  const Nbhd nb(d, x, y, z);
+  const FieldAt<float> U{u, &nb};
+  const CoefAt Bc{cf, &nb};
+  const long long i = nb(0, 0, 0);
+  out[i] = r[i] - op_h2<float>(U, Bc, form) * inv_h2 / cf.J[i];
 }
 
 // Weighted Jacobi (Appendix B, Eq. jacobi): e' = e + omega (r - L e) / D_L, D_L = diag(M) / J,
-// written as e + omega (J r - M e) / diag(M).
-template <typename T>
-__global__ void k_curv_jacobi(Dims d, CurvCoef cf, const T* __restrict__ r, const T* __restrict__ e_in,
-                              T* __restrict__ e_out, int form, T omega) {
+// written as e + omega (J r - M e) / diag(M) with the h^2 scalings cancelling; D = h^2 diag(M)
+// is built once per geometry (k_curv_diag).
+__device__ __forceinline__ float jacobi_value(float e, float r, float J, float D, float Mh2, float h2, float omega) {
+  return __fmaf_rn(omega, __fdiv_rn(__fmaf_rn(__fmul_rn(J, r), h2, -Mh2), D), e);
+}
+__global__ void k_curv_jacobi(Dims d, CurvCoef cf, const float* __restrict__ r, const float* __restrict__ e_in,
+                              float* __restrict__ e_out, int form, float omega) {
   const int x = blockIdx.x * BX + threadIdx.x, y = blockIdx.y * BY + threadIdx.y, z = blockIdx.z;
   if (x >= d.nx || y >= d.ny) return;
   const Nbhd nb(d, x, y, z);
-  const FieldAt<T> U{e_in, &nb};
+  const FieldAt<float> U{e_in, &nb};
   const CoefAt Bc{cf, &nb};
   const long long i = nb(0, 0, 0);
-  const T Mh2 = op_h2<T>(U, Bc, form);
-  const T Dh2 = diag_form_h2<T>(Bc, form);
-  // (J r - M e) / diag(M) with h^2 scalings cancelling: (J r h^2 - M e h^2) / (diag h^2)
-  e_out[i] = e_in[i] + omega * ((T(cf.J[i]) * r[i] * cf.h2 - Mh2) / Dh2);
+  e_out[i] = jacobi_value(e_in[i], r[i], cf.J[i], cf.D[i], op_h2<float>(U, Bc, form), cf.h2, omega);
+}
+
+__global__ void k_curv_diag(Dims d, CurvCoef cf, int form, float* __restrict__ D) {
+  const int x = blockIdx.x * BX + threadIdx.x, y = blockIdx.y * BY + threadIdx.y, z = blockIdx.z;
+  if (x >= d.nx || y >= d.ny) return;
+  const Nbhd nb(d, x, y, z);
+  const CoefAt Bc{cf, &nb};
+  D[nb(0, 0, 0)] = diag_form_h2<float>(Bc, form);
 }
 
 // The first weighted-Jacobi sweep of a smoothing pass that starts from e = 0: op(0) = 0,
-// so the sweep is pointwise, e' = omega (J r h^2 - 0) / diag h^2, and reads only r, J and
-// the coefficients of the diagonal.  Written with the sweep's own expression, an explicit
-// zero iterate and operator value, so that it rounds exactly like k_curv_tiled<CM_JACOBI>
-// on a zero input (whose operator sum is +0).
-template <int FORM>
-__global__ void k_curv_jacobi_zero(Dims d, CurvCoef cf, const float* __restrict__ r, float* __restrict__ e_out,
-                                   float omega) {
-  const int x = blockIdx.x * BX + threadIdx.x, y = blockIdx.y * BY + threadIdx.y, z = blockIdx.z;
-  if (x >= d.nx || y >= d.ny) return;
-  const Nbhd nb(d, x, y, z);
-  const CoefAt Bc{cf, &nb};
-  const long long i = nb(0, 0, 0);
-  const float Dh2 = FORM == 2 ? diag_S_h2<float>(Bc) : diag_M_h2<float>(Bc);
-  const float Jc = cf.J[i], rc = r[i];
-  const float u0 = 0.f, Mh2 = 0.f;
-  e_out[i] = u0 + omega * ((Jc * rc * cf.h2 - Mh2) / Dh2);
+// so the sweep is pointwise, rounded as in the sweeps of a zero array.
+__global__ void k_curv_jacobi_zero(long long n, const float* __restrict__ J, const float* __restrict__ D, float h2,
+                                   float omega, const float* __restrict__ r, float* __restrict__ e_out) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+    e_out[i] = jacobi_value(0.f, r[i], J[i], D[i], 0.f, h2, omega);
 }
 
 // Dense matrix of the level operator (row-major n x n, FP64): entry (i, j) = (op(e_j) / J)_i.
@@ -980,14 +966,14 @@ dim3 curv_tiled_grid(Dims d) {
 
 enum CurvMode { CM_JACOBI = 0, CM_RESID = 1 };
 
-// FP32 forms.  CM_JACOBI: out = e + omega (J r h^2 - op(e) h^2) / diag h^2 (Appendix B);
-// CM_RESID: out = r - op(u) / (h^2 J) with block partial sums of out^2 (partials nullable).
+// FP32 forms, for what the z-marching kernels of curv_march.cu do not take (rows or fields
+// off 16 bytes).  CM_JACOBI: out = e + omega (J r h^2 - op(e) h^2) / D (Appendix B);
+// CM_RESID: out = r - op(u) / (h^2 J).
 template <int MODE, int TR>
 __global__ void __launch_bounds__(CNT) k_curv_tiled(Dims d, CurvCoef cf, const float* __restrict__ r,
                                                       const float* __restrict__ u, float* __restrict__ out,
-                                                      float omega, float inv_h2, double* __restrict__ partials, int zc) {
+                                                      float omega, float inv_h2, int zc) {
   extern __shared__ __align__(16) char smc[];
-  __shared__ double shr[32];
   const Ring<float> ring{smc};
   const int tx = threadIdx.x % CTX, ty = threadIdx.x / CTX;
   const int x0 = blockIdx.x * CTX, y0 = blockIdx.y * CTY, z0 = blockIdx.z * zc;
@@ -996,7 +982,6 @@ __global__ void __launch_bounds__(CNT) k_curv_tiled(Dims d, CurvCoef cf, const f
   const bool own = x < d.nx && y < d.ny;
   const long long pst = (long long)d.nx * d.ny;
   const int c = (ty + 1) * CSW + tx + 1;
-  float rr = 0.f;
   __shared__ float sfx[CTY][CTX + 1], sfy[CTY + 1][CTX];  // x- and y-face fluxes of M (form 0)
   float fzm = 0.f;                                         // -z face flux of M (form 0)
   PlaneRegs<float> R;
@@ -1007,22 +992,22 @@ __global__ void __launch_bounds__(CNT) k_curv_tiled(Dims d, CurvCoef cf, const f
   load_plane(d, u, cf, PI, z0, R);
   store_plane(ring, slot(z0), R);
   load_plane(d, u, cf, PI, z0 + 1, R);
-  // J and r of the thread's cell, one plane ahead
+  // J, D and r of the thread's cell, one plane ahead
   const long long i0 = (long long)y * d.nx + x;
-  float Jn = 0.f, rn = 0.f;
-  if (own) {
-    Jn = cf.J[(long long)z0 * pst + i0];
-    rn = r[(long long)z0 * pst + i0];
-  }
+  float Jn = 0.f, Dn = 0.f, rn = 0.f;
+  auto fetch = [&](int z) {
+    const long long i = (long long)z * pst + i0;
+    Jn = cf.J[i];
+    if (MODE == CM_JACOBI) Dn = cf.D[i];
+    rn = r[i];
+  };
+  if (own) fetch(z0);
   for (int t = z0; t < zend; ++t) {
     store_plane(ring, slot(t + 1), R);
     __syncthreads();
     if (t + 1 < zend) load_plane(d, u, cf, PI, t + 2, R);
-    const float Jc = Jn, rc = rn;
-    if (own && t + 1 < zend) {
-      Jn = cf.J[(long long)(t + 1) * pst + i0];
-      rn = r[(long long)(t + 1) * pst + i0];
-    }
+    const float Jc = Jn, Dc = Dn, rc = rn;
+    if (own && t + 1 < zend) fetch(t + 1);
     const RingU<float> U{{ring.u(slot(t - 1)), ring.u(slot(t)), ring.u(slot(t + 1))}, c};
     const RingB Bc{{ring.b(slot(t - 1)), ring.b(slot(t)), ring.b(slot(t + 1))}, c};
     float Mh2 = 0.f;
@@ -1050,19 +1035,8 @@ __global__ void __launch_bounds__(CNT) k_curv_tiled(Dims d, CurvCoef cf, const f
     if (own) {
       const long long i = (long long)t * pst + i0;
       if constexpr (TR != 0) Mh2 = TR == 2 ? apply_S_h2<float>(U, Bc) : apply_MT_h2<float>(U, Bc);
-      if (MODE == CM_JACOBI) {
-        const float Dh2 = TR == 2 ? diag_S_h2<float>(Bc) : diag_M_h2<float>(Bc);
-        out[i] = U(0, 0, 0) + omega * ((Jc * rc * cf.h2 - Mh2) / Dh2);
-      } else {
-        const float res = rc - Mh2 * inv_h2 / Jc;
-        out[i] = res;
-        rr += res * res;
-      }
+      out[i] = MODE == CM_JACOBI ? jacobi_value(U(0, 0, 0), rc, Jc, Dc, Mh2, cf.h2, omega) : rc - Mh2 * inv_h2 / Jc;
     }
-  }
-  if (MODE == CM_RESID && partials) {
-    const double s = block_sum_f(rr, shr);
-    if (is_thread0()) partials[block_linear_id()] = s;
   }
 }
 
@@ -1224,57 +1198,57 @@ long long curv_partial_count(Dims d) {
 
 // FP32 sweeps and residuals of levels of at most 32^3 cells run one thread per cell
 // (k_curv_jacobi / k_curv_residual: every load of a cell in one round) instead of the
-// z-streaming tiles, whose few CTAs there take one dependent round of loads per plane.
-// Both evaluate the same operator templates in the same order, so the results are the
-// same bits (the moving-mesh solve's phi, delta-bar and psi-bar were compared).
+// marching tiles, whose few CTAs there take one dependent round of loads per plane.
 static bool curv_cellwise(Dims d) { return (long long)d.nx * d.ny * d.nz <= 32 * 32 * 32; }
 
-template <typename T>
-cudaError_t launch_curv_residual(cudaStream_t st, Dims d, CurvCoef cf, const T* r, const T* u, T* out, int form,
-                                 double* partials) {
-  if (form < 0 || form > 2) return cudaErrorInvalidValue;
-  if (sizeof(T) == 4 && !partials && curv_cellwise(d)) {
-    k_curv_residual<T><<<cell_grid(d), dim3(BX, BY), 0, st>>>(d, cf, r, u, out, (T)(1.0 / cf.h2), form, partials);
-  } else if constexpr (sizeof(T) == 4) {
-    const size_t sm = 4 * ring_slot_bytes<float>();
-    const float ih2 = (float)(1.0 / cf.h2);
-    const dim3 g = curv_tiled_grid(d);
-    const int zc = curv_zchunk(d);
-    if (form == 2) k_curv_tiled<CM_RESID, 2><<<g, CNT, sm, st>>>(d, cf, r, u, out, 0.f, ih2, partials, zc);
-    else if (form == 1) k_curv_tiled<CM_RESID, 1><<<g, CNT, sm, st>>>(d, cf, r, u, out, 0.f, ih2, partials, zc);
-    else k_curv_tiled<CM_RESID, 0><<<g, CNT, sm, st>>>(d, cf, r, u, out, 0.f, ih2, partials, zc);
-  } else {
-    k_curv_residual<T><<<cell_grid(d), dim3(BX, BY), 0, st>>>(d, cf, r, u, out, (T)(1.0 / cf.h2), form, partials);
-  }
+cudaError_t launch_curv_diag(cudaStream_t st, Dims d, const CurvCoef& cf, int form, float* D) {
+  k_curv_diag<<<cell_grid(d), dim3(BX, BY), 0, st>>>(d, cf, form, D);
   note_launch();
   return cudaGetLastError();
 }
 
-template <typename T>
-cudaError_t launch_curv_jacobi(cudaStream_t st, Dims d, CurvCoef cf, const T* r, const T* e_in, T* e_out, int form,
-                               T omega) {
-  if (form < 0 || form > 2) return cudaErrorInvalidValue;
-  if (sizeof(T) == 4 && curv_cellwise(d)) {
-    k_curv_jacobi<T><<<cell_grid(d), dim3(BX, BY), 0, st>>>(d, cf, r, e_in, e_out, form, omega);
-  } else if constexpr (sizeof(T) == 4) {
-    const size_t sm = 4 * ring_slot_bytes<float>();
-    const dim3 g = curv_tiled_grid(d);
-    const int zc = curv_zchunk(d);
-    if (form == 2) k_curv_tiled<CM_JACOBI, 2><<<g, CNT, sm, st>>>(d, cf, r, e_in, e_out, omega, 0.f, nullptr, zc);
-    else if (form == 1) k_curv_tiled<CM_JACOBI, 1><<<g, CNT, sm, st>>>(d, cf, r, e_in, e_out, omega, 0.f, nullptr, zc);
-    else k_curv_tiled<CM_JACOBI, 0><<<g, CNT, sm, st>>>(d, cf, r, e_in, e_out, omega, 0.f, nullptr, zc);
-  } else {
-    k_curv_jacobi<T><<<cell_grid(d), dim3(BX, BY), 0, st>>>(d, cf, r, e_in, e_out, form, omega);
-  }
+template <int MODE>
+static cudaError_t launch_tiled(cudaStream_t st, Dims d, const CurvCoef& cf, const float* r, const float* u,
+                                float* out, int form, float omega) {
+  const size_t sm = 4 * ring_slot_bytes<float>();
+  const float ih2 = (float)(1.0 / cf.h2);
+  const dim3 g = curv_tiled_grid(d);
+  const int zc = curv_zchunk(d);
+  if (form == 2) k_curv_tiled<MODE, 2><<<g, CNT, sm, st>>>(d, cf, r, u, out, omega, ih2, zc);
+  else if (form == 1) k_curv_tiled<MODE, 1><<<g, CNT, sm, st>>>(d, cf, r, u, out, omega, ih2, zc);
+  else k_curv_tiled<MODE, 0><<<g, CNT, sm, st>>>(d, cf, r, u, out, omega, ih2, zc);
   note_launch();
   return cudaGetLastError();
 }
 
-cudaError_t launch_curv_jacobi_zero(cudaStream_t st, Dims d, CurvCoef cf, const float* r, float* e_out, int form,
+cudaError_t launch_curv_residual(cudaStream_t st, Dims d, const CurvCoef& cf, const float* r, const float* u,
+                                 float* out, int form) {
+  if (form < 0 || form > 2) return cudaErrorInvalidValue;
+  if (curv_cellwise(d)) {
+    k_curv_residual<<<cell_grid(d), dim3(BX, BY), 0, st>>>(d, cf, r, u, out, (float)(1.0 / cf.h2), form);
+    note_launch();
+    return cudaGetLastError();
+  }
+  if (curv_march_ok(d, cf, u)) return launch_march_residual(st, d, cf, r, u, out, form);
+  return launch_tiled<CM_RESID>(st, d, cf, r, u, out, form, 0.f);
+}
+
+cudaError_t launch_curv_jacobi(cudaStream_t st, Dims d, const CurvCoef& cf, const float* r, const float* e_in,
+                               float* e_out, int form, float omega) {
+  if (form < 0 || form > 2) return cudaErrorInvalidValue;
+  if (curv_cellwise(d)) {
+    k_curv_jacobi<<<cell_grid(d), dim3(BX, BY), 0, st>>>(d, cf, r, e_in, e_out, form, omega);
+    note_launch();
+    return cudaGetLastError();
+  }
+  if (curv_march_ok(d, cf, e_in)) return launch_march_jacobi(st, d, cf, r, e_in, e_out, form, omega);
+  return launch_tiled<CM_JACOBI>(st, d, cf, r, e_in, e_out, form, omega);
+}
+
+cudaError_t launch_curv_jacobi_zero(cudaStream_t st, Dims d, const CurvCoef& cf, const float* r, float* e_out,
                                     float omega) {
-  if (form < 0 || form > 2) return cudaErrorInvalidValue;
-  if (form == 2) k_curv_jacobi_zero<2><<<cell_grid(d), dim3(BX, BY), 0, st>>>(d, cf, r, e_out, omega);
-  else k_curv_jacobi_zero<0><<<cell_grid(d), dim3(BX, BY), 0, st>>>(d, cf, r, e_out, omega);
+  const long long n = ncell(d);
+  k_curv_jacobi_zero<<<(int)df_partial_count(n), 256, 0, st>>>(n, cf.J, cf.D, cf.h2, omega, r, e_out);
   note_launch();
   return cudaGetLastError();
 }
@@ -1309,9 +1283,5 @@ cudaError_t launch_ratio(cudaStream_t st, const double* a, const double* b, doub
 
 template cudaError_t launch_curv_apply<float>(cudaStream_t, Dims, CurvCoef, const float*, float*, int, int);
 template cudaError_t launch_curv_apply<double>(cudaStream_t, Dims, CurvCoef, const double*, double*, int, int);
-template cudaError_t launch_curv_residual<float>(cudaStream_t, Dims, CurvCoef, const float*, const float*, float*, int, double*);
-template cudaError_t launch_curv_residual<double>(cudaStream_t, Dims, CurvCoef, const double*, const double*, double*, int, double*);
-template cudaError_t launch_curv_jacobi<float>(cudaStream_t, Dims, CurvCoef, const float*, const float*, float*, int, float);
-template cudaError_t launch_curv_jacobi<double>(cudaStream_t, Dims, CurvCoef, const double*, const double*, double*, int, double);
 
 }  // namespace gbmg

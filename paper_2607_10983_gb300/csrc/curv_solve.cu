@@ -25,28 +25,18 @@ enum CurvScal { S_SUMJ = 6, S_MW = 9, S_SLAM = 10 };
 // operator form of the forward (tr false) or transposed (tr true) problem: 0 = M, 1 = M^T, 2 = S
 int curv_form(const gbmg_ctx* c, bool tr) { return c->o.curv_sym ? 2 : (tr ? 1 : 0); }
 
-template <typename T>
-const T* curv_G(const gbmg_ctx* c, bool tr);
-template <>
-const float* curv_G<float>(const gbmg_ctx* c, bool tr) { return tr ? c->G32T : c->G32; }
-template <>
-const double* curv_G<double>(const gbmg_ctx* c, bool tr) { return tr ? c->G64T : c->G64; }
-
 // nu weighted-Jacobi sweeps; from_zero: the iterate is zero, so the first sweep is the
 // pointwise one (no read of e; the same values as a full sweep of zeros)
-template <typename T>
-gbmg_status curv_smooth(gbmg_ctx* c, int l, T*& e, T*& eo, const T* r, int nu, bool tr, bool from_zero) {
+gbmg_status curv_smooth(gbmg_ctx* c, int l, float*& e, float*& eo, const float* r, int nu, bool tr, bool from_zero) {
   const Level& L = c->lv[l];
   for (int k = 0; k < nu; ++k) {
     if (k == 0 && from_zero) {
-      if constexpr (sizeof(T) == 4) {
-        TRY(launch_curv_jacobi_zero(c->stream, L.d, L.cc, r, eo, curv_form(c, tr), (float)c->o.omega));
-        std::swap(e, eo);
-        continue;
-      }
+      TRY(launch_curv_jacobi_zero(c->stream, L.d, L.cc, r, eo, (float)c->o.omega));
+      std::swap(e, eo);
+      continue;
     }
     ProfScope ps(c, l == 0 ? GBMG_PROF_CURV0 : GBMG_PROF_OFF);
-    TRY(launch_curv_jacobi<T>(c->stream, L.d, L.cc, r, e, eo, curv_form(c, tr), (T)c->o.omega));
+    TRY(launch_curv_jacobi(c->stream, L.d, L.cc, r, e, eo, curv_form(c, tr), (float)c->o.omega));
     std::swap(e, eo);
   }
   return GBMG_OK;
@@ -56,23 +46,23 @@ gbmg_status curv_smooth(gbmg_ctx* c, int l, T*& e, T*& eo, const T* r, int nu, b
 // per operation (Sec. 4.3, Eq. curv_error; Appendix B), from e = 0: the iterate's
 // content is not read when nu1 > 0 (the first sweep is the pointwise one), and must be
 // zero otherwise.
-template <typename T>
-gbmg_status vcycle_curv(gbmg_ctx* c, int l, T*& e, T*& eo, const T* r, bool tr) {
+gbmg_status vcycle_curv(gbmg_ctx* c, int l, float*& e, float*& eo, const float* r, bool tr) {
   const Level& L = c->lv[l];
   if (l == c->L - 1) {
-    TRY(launch_coarse_matvec<T>(c->stream, c->nc, curv_G<T>(c, tr), r, e));
+    TRY(launch_coarse_matvec<float>(c->stream, c->nc, tr ? c->G32T : c->G32, r, e));
     return GBMG_OK;
   }
-  TRYS(curv_smooth<T>(c, l, e, eo, r, c->o.nu1, tr, true));
-  TRY(launch_curv_residual<T>(c->stream, L.d, L.cc, r, e, (T*)L.t, curv_form(c, tr), nullptr));
+  TRYS(curv_smooth(c, l, e, eo, r, c->o.nu1, tr, true));
+  TRY(launch_curv_residual(c->stream, L.d, L.cc, r, e, (float*)L.t, curv_form(c, tr)));
   const Level& C = c->lv[l + 1];
-  TRY(launch_restrict<T>(c->stream, L.d, (const T*)L.t, (T*)C.r));
-  T* ce = (T*)C.e;
-  T* ceo = (T*)C.e2;
-  if (l + 1 < c->L - 1 && c->o.nu1 == 0) TRY(cudaMemsetAsync(ce, 0, (size_t)ncell(C.d) * sizeof(T), c->stream));
-  TRYS(vcycle_curv<T>(c, l + 1, ce, ceo, (const T*)C.r, tr));
-  TRY(launch_prolong_add<T>(c->stream, C.d, ce, e));
-  TRYS(curv_smooth<T>(c, l, e, eo, r, c->o.nu2, tr, false));
+  TRY(launch_restrict<float>(c->stream, L.d, (const float*)L.t, (float*)C.r));
+  float* ce = (float*)C.e;
+  float* ceo = (float*)C.e2;
+  if (l + 1 < c->L - 1 && c->o.nu1 == 0)
+    TRY(cudaMemsetAsync(ce, 0, (size_t)ncell(C.d) * sizeof(float), c->stream));
+  TRYS(vcycle_curv(c, l + 1, ce, ceo, (const float*)C.r, tr));
+  TRY(launch_prolong_add<float>(c->stream, C.d, ce, e));
+  TRYS(curv_smooth(c, l, e, eo, r, c->o.nu2, tr, false));
   return GBMG_OK;
 }
 
@@ -91,7 +81,7 @@ gbmg_status curv_cycle(gbmg_ctx* c, bool tr, float* r0) {
   float* e = (float*)L0.e;
   float* eo = (float*)L0.e2;
   if (c->o.nu1 == 0) TRY(cudaMemsetAsync(e, 0, (size_t)n * sizeof(float), c->stream));
-  TRYS(vcycle_curv<float>(c, 0, e, eo, r0, tr));
+  TRYS(vcycle_curv(c, 0, e, eo, r0, tr));
   TRY(launch_df_update(c->stream, n, c->phi_df, e, nullptr));
   {
     ProfScope ps(c, GBMG_PROF_DF0);
@@ -183,6 +173,15 @@ gbmg_status gbmg::curv_solve(gbmg_ctx* c, const double* F, double* phi, double t
 
 namespace {
 
+// The operator's diagonal on every level that is smoothed.
+gbmg_status build_diag(gbmg_ctx* c) {
+  for (int l = 0; l + 1 < c->L; ++l) {
+    const Level& L = c->lv[l];
+    TRY(launch_curv_diag(c->stream, L.d, L.cc, curv_form(c, false), (float*)L.cc.D));
+  }
+  return GBMG_OK;
+}
+
 // Exact inverses of the coarsest operator and of its transposed-solve twin (minimum-norm,
 // left null vector J), built from the coarsest level's coefficients.  Waits for the stream.
 gbmg_status build_coarsest(gbmg_ctx* c, const char* who) {
@@ -225,6 +224,7 @@ extern "C" gbmg_status mg_set_geometry(gbmg_ctx* c, const double* psi_dev) {
     for (int k = 0; k < 6; ++k) o.B[k] = (float*)L.cc.B[k];
     TRY(launch_geom(c->stream, L.d, L.psi, L.h, o));
   }
+  TRYS(build_diag(c));
   TRYS(build_coarsest(c, "mg_set_geometry"));
   c->geom_ready = true;
   c->geom_from_psi = true;
@@ -251,6 +251,7 @@ extern "C" gbmg_status mg_set_coefficients(gbmg_ctx* c, const float* J_dev, cons
       for (int k = 0; k < 6; ++k) TRY(launch_restrict<float>(c->stream, F.d, F.cc.B[k], (float*)L.cc.B[k]));
     }
   }
+  TRYS(build_diag(c));
   TRYS(build_coarsest(c, "mg_set_coefficients"));
   c->geom_ready = true;
   return GBMG_OK;
@@ -334,7 +335,7 @@ extern "C" gbmg_status mg_curv_residual(gbmg_ctx* c, int level, int transpose, c
   TRYS(curv_component_check(c, level, r, u, out, "mg_curv_residual"));
   DeviceGuard g(c->device);
   const Level& L = c->lv[level];
-  TRY(launch_curv_residual<float>(c->stream, L.d, L.cc, r, u, out, curv_form(c, transpose != 0), nullptr));
+  TRY(launch_curv_residual(c->stream, L.d, L.cc, r, u, out, curv_form(c, transpose != 0)));
   return GBMG_OK;
 }
 
@@ -345,8 +346,8 @@ extern "C" gbmg_status mg_curv_smooth(gbmg_ctx* c, int level, int transpose, con
   DeviceGuard g(c->device);
   const Level& L = c->lv[level];
   const int form = curv_form(c, transpose != 0);
-  if (e_in) TRY(launch_curv_jacobi<float>(c->stream, L.d, L.cc, r, e_in, e_out, form, (float)c->o.omega));
-  else TRY(launch_curv_jacobi_zero(c->stream, L.d, L.cc, r, e_out, form, (float)c->o.omega));
+  if (e_in) TRY(launch_curv_jacobi(c->stream, L.d, L.cc, r, e_in, e_out, form, (float)c->o.omega));
+  else TRY(launch_curv_jacobi_zero(c->stream, L.d, L.cc, r, e_out, (float)c->o.omega));
   return GBMG_OK;
 }
 
@@ -372,7 +373,7 @@ extern "C" gbmg_status mg_curv_vcycle(gbmg_ctx* c, int transpose, const float* r
   float* e = (float*)L0.e;
   float* eo = (float*)L0.e2;
   TRY(cudaMemsetAsync(e, 0, (size_t)n * 4, c->stream));
-  TRYS(vcycle_curv<float>(c, 0, e, eo, r, transpose != 0));
+  TRYS(vcycle_curv(c, 0, e, eo, r, transpose != 0));
   TRY(cudaMemcpyAsync(e_out, e, (size_t)n * 4, cudaMemcpyDeviceToDevice, c->stream));
   return GBMG_OK;
 }

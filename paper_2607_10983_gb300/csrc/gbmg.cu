@@ -172,7 +172,7 @@ extern "C" gbmg_status mg_setup(gbmg_ctx** out, int nx, int ny, int nz, int leve
     lo[l] = Offs{take(b), take(b), take(b), take(b), take(b)};
     if (curv) {
       lpsi[l] = take((size_t)ncell(dims[l]) * sizeof(double));
-      lcoef[l] = take((size_t)ncell(dims[l]) * 7 * sizeof(float));
+      lcoef[l] = take((size_t)ncell(dims[l]) * 8 * sizeof(float));
     }
   }
   size_t oF = 0, oP = 0, oP2 = 0, oR = 0;
@@ -223,6 +223,7 @@ extern "C" gbmg_status mg_setup(gbmg_ctx** out, int nx, int ny, int nz, int leve
       const long long nl = ncell(dims[l]);
       L.cc.J = cb;
       for (int k = 0; k < 6; ++k) L.cc.B[k] = cb + (k + 1) * nl;
+      L.cc.D = cb + 7 * nl;
       L.cc.h2 = (float)(L.h * L.h);
     }
   }

@@ -113,9 +113,11 @@ cudaError_t launch_df_update_residual(cudaStream_t st, Dims d, const float2* phi
 
 // ---- curvilinear operator (moving mesh) ----
 // Per-level geometry: J = det A and the packed symmetric B = J A^-2 (xx, yy, zz, xy, xz, yz).
+// D: h^2 times the operator's diagonal (of the context's discretisation).
 struct CurvCoef {
   const float* J;
   const float* B[6];
+  const float* D;
   float h2;  // h_l^2
 };
 struct CurvCoefOut {
@@ -128,20 +130,27 @@ cudaError_t launch_geom(cudaStream_t st, Dims d, const double* psi, double h, Cu
 // out = op(u) (/ J when divide_J)
 template <typename T>
 cudaError_t launch_curv_apply(cudaStream_t st, Dims d, CurvCoef cf, const T* u, T* out, int form, int divide_J);
-// out = r - op(u) / J; partials (nullable): block sums of out^2
-template <typename T>
-cudaError_t launch_curv_residual(cudaStream_t st, Dims d, CurvCoef cf, const T* r, const T* u, T* out, int form,
-                                 double* partials);
-template <typename T>
-cudaError_t launch_curv_jacobi(cudaStream_t st, Dims d, CurvCoef cf, const T* r, const T* e_in, T* e_out, int form,
-                               T omega);
-// dense n x n matrix of op / J on a (small) level, FP64 row-major
-// e_out = the weighted-Jacobi sweep of an iterate that is zero (pointwise; FP32)
-cudaError_t launch_curv_jacobi_zero(cudaStream_t st, Dims d, CurvCoef cf, const float* r, float* e_out, int form,
+// out = r - op(u) / J, FP32
+cudaError_t launch_curv_residual(cudaStream_t st, Dims d, const CurvCoef& cf, const float* r, const float* u,
+                                 float* out, int form);
+// D of a level from its B (form 2: the symmetric variant's diagonal)
+cudaError_t launch_curv_diag(cudaStream_t st, Dims d, const CurvCoef& cf, int form, float* D);
+// e_out = a weighted-Jacobi sweep of e_in, FP32
+cudaError_t launch_curv_jacobi(cudaStream_t st, Dims d, const CurvCoef& cf, const float* r, const float* e_in,
+                               float* e_out, int form, float omega);
+// e_out = the sweep of an iterate that is zero (pointwise; FP32)
+cudaError_t launch_curv_jacobi_zero(cudaStream_t st, Dims d, const CurvCoef& cf, const float* r, float* e_out,
                                     float omega);
+// the z-marching kernels: nx a multiple of 4, u and B on 16 bytes
+bool curv_march_ok(Dims d, const CurvCoef& cf, const float* u);
+cudaError_t launch_march_jacobi(cudaStream_t st, Dims d, const CurvCoef& cf, const float* r, const float* e_in,
+                                float* e_out, int form, float omega);
+cudaError_t launch_march_residual(cudaStream_t st, Dims d, const CurvCoef& cf, const float* r, const float* u,
+                                  float* out, int form);
+// dense n x n matrix of op / J on a (small) level, FP64 row-major
 cudaError_t launch_curv_dense(cudaStream_t st, Dims d, CurvCoef cf, int form, double* out);
 // double-float outer residual: r = b - op(u)/J with b = J (src - m) (scale_J) or src
-// block partial sums written by launch_curv_df_residual and launch_curv_residual<float>
+// block partial sums written by launch_curv_df_residual
 long long curv_partial_count(Dims d);
 cudaError_t launch_curv_df_residual(cudaStream_t st, Dims d, CurvCoef cf, const float2* src, const double* m_dev,
                                     int scale_J, const float2* u, int form, float* r, double* pr2, double* pf2);
