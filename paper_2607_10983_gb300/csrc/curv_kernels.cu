@@ -322,6 +322,56 @@ __global__ void k_curv_jacobi_zero(long long n, const float* __restrict__ J, con
     e_out[i] = jacobi_value(0.f, r[i], J[i], D[i], 0.f, h2, omega);
 }
 
+// Full weighting to a coarse level and the first sweep of its pre-smoothing, from zero: one
+// thread per coarse column of zc planes.  The weights run along z first, then y, then x
+// (k_restrict's order and bits); a thread reads each fine plane once, as one x-pair and one
+// odd cell per row, 12 loads per coarse cell instead of 27.  256^3: 35 -> 18 us, and the
+// sweep's own pass over r, J and D is gone.
+__global__ void k_curv_restrict(Dims df, const float* __restrict__ f, float* __restrict__ rc, float* __restrict__ e1,
+                                const float* __restrict__ J, const float* __restrict__ D, float h2, float omega, int zc) {
+  const Dims dc{df.nx / 2, df.ny / 2, df.nz / 2};
+  const int X = blockIdx.x * BX + threadIdx.x, Y = blockIdx.y * BY + threadIdx.y;
+  if (X >= dc.nx || Y >= dc.ny) return;
+  const int Z0 = blockIdx.z * zc, Z1 = min(Z0 + zc, dc.nz);
+  const long long pst = (long long)df.nx * df.ny;
+  int row[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) row[k] = wrapi(2 * Y + k - 1, df.ny) * df.nx;
+  const int xm = wrapi(2 * X - 1, df.nx);
+  struct Plane {
+    float v[3][3];  // [row][x - 1, x, x + 1]
+  };
+  auto load = [&](int z, Plane& p) {
+    const float* q = f + wrapi(z, df.nz) * pst;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const float2 c = __ldg(reinterpret_cast<const float2*>(q + row[k] + 2 * X));
+      p.v[k][0] = __ldg(q + row[k] + xm);
+      p.v[k][1] = c.x;
+      p.v[k][2] = c.y;
+    }
+  };
+  Plane a, b, c;
+  load(2 * Z0 - 1, a);
+  for (int Z = Z0; Z < Z1; ++Z) {
+    load(2 * Z, b);
+    load(2 * Z + 1, c);
+    float yv[3];
+#pragma unroll
+    for (int x = 0; x < 3; ++x) {
+      float zv[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) zv[k] = fw3(a.v[k][x], b.v[k][x], c.v[k][x]);
+      yv[x] = fw3(zv[0], zv[1], zv[2]);
+    }
+    const float v = fw3(yv[0], yv[1], yv[2]);
+    const long long i = lin(dc, X, Y, Z);
+    rc[i] = v;
+    if (e1) e1[i] = jacobi_value(0.f, v, J[i], D[i], 0.f, h2, omega);
+    a = c;
+  }
+}
+
 // Dense matrix of the level operator (row-major n x n, FP64): entry (i, j) = (op(e_j) / J)_i.
 struct UnitAt {
   const Nbhd* nb;
@@ -601,10 +651,11 @@ __device__ __forceinline__ PlaneIdx plane_idx(Dims d, int x0, int y0) {
   return P;
 }
 
-// Plane z in [-1, nz] (the chunk's planes and one on each side) wrapped onto the mesh.
+// Plane z in [-1, nz] (the chunk's planes and one on each side) wrapped onto the mesh; of
+// u + e (double-float plus FP32) when e is given.
 template <typename V>
 __device__ __forceinline__ void load_plane(Dims d, const V* __restrict__ u, const CurvCoef& cf, const PlaneIdx& P,
-                                           int z, PlaneRegs<V>& R) {
+                                           int z, PlaneRegs<V>& R, const float* __restrict__ e = nullptr) {
   const int zw = z < 0 ? z + d.nz : (z >= d.nz ? z - d.nz : z);
   const long long zo = (long long)zw * d.nx * d.ny;
 #pragma unroll
@@ -613,6 +664,8 @@ __device__ __forceinline__ void load_plane(Dims d, const V* __restrict__ u, cons
     if (q < CSN) {
       const long long gi = zo + P.off[k];
       R.u[k] = u[gi];
+      if constexpr (sizeof(V) == 8)
+        if (e) R.u[k] = df_add_f(R.u[k], __ldg(e + gi));
 #pragma unroll
       for (int m = 0; m < 6; ++m) R.b[k][m] = __ldg(cf.B[m] + gi);
     }
@@ -1046,15 +1099,21 @@ struct DfRingAt {
   __device__ __forceinline__ float2 operator()(int dx, int dy, int dz) const { return pl[dz + 1][c + dy * CSW + dx]; }
 };
 
-// r = (b - op(u) / h^2) / J rounded to float, with b = J (src - m) when scale_J (forward
-// source in L-form) or b = src (transposed solve, M-form right-hand side).  Partial sums
-// of r^2 and of (b / J)^2.  Three CTAs per SM (80 registers, no spill): the kernel is
+// One defect-correction step of the finest level: u' = u + e (e NULL: u' = u, not written),
+// r = (b - op(u') / h^2) / J rounded to float, with b = J (src - m) when scale_J (forward
+// source in L-form) or b = src (transposed solve, M-form right-hand side), and e1 (nullable)
+// = the first weighted-Jacobi sweep of the next cycle, from zero.  Partial sums of r^2 and of
+// (b / J)^2.  Updating and sweeping here saves their own passes over u, e, r, J and the
+// diagonal.  For meshes whose rows the z-marching kernel (curv_march_df.cu) cannot copy.  Three CTAs per SM (80 registers, no spill): the kernel is
 // bound by instruction issue, and 24 warps per SM run it 6% faster than 16.
 __global__ void __launch_bounds__(CNT, 3) k_curv_df_residual_tiled(Dims d, CurvCoef cf, const float2* __restrict__ src,
                                                                  const double* __restrict__ m_dev, int scale_J,
-                                                                 const float2* __restrict__ u, int form,
-                                                                 float* __restrict__ r, double* __restrict__ pr2,
-                                                                 double* __restrict__ pf2, int zc) {
+                                                                 const float2* __restrict__ u,
+                                                                 const float* __restrict__ e, float2* __restrict__ u_out,
+                                                                 int form, float* __restrict__ r,
+                                                                 float* __restrict__ e1, float omega,
+                                                                 double* __restrict__ pr2, double* __restrict__ pf2,
+                                                                 int zc) {
   extern __shared__ __align__(16) char smc[];
   __shared__ double shr[32];
   const Ring<float2> ring{smc};
@@ -1073,11 +1132,11 @@ __global__ void __launch_bounds__(CNT, 3) k_curv_df_residual_tiled(Dims d, CurvC
   PlaneRegs<float2> R;
   const PlaneIdx PI = plane_idx(d, x0, y0);
   auto slot = [&](int p) { return (p - (z0 - 1)) & 3; };
-  load_plane(d, u, cf, PI, z0 - 1, R);
+  load_plane(d, u, cf, PI, z0 - 1, R, e);
   store_plane(ring, slot(z0 - 1), R);
-  load_plane(d, u, cf, PI, z0, R);
+  load_plane(d, u, cf, PI, z0, R, e);
   store_plane(ring, slot(z0), R);
-  load_plane(d, u, cf, PI, z0 + 1, R);
+  load_plane(d, u, cf, PI, z0 + 1, R, e);
   // J and the source of the thread's cell, one plane ahead
   const long long i0 = (long long)y * d.nx + x;
   float Jn = 0.f;
@@ -1089,7 +1148,7 @@ __global__ void __launch_bounds__(CNT, 3) k_curv_df_residual_tiled(Dims d, CurvC
   for (int t = z0; t < zend; ++t) {
     store_plane(ring, slot(t + 1), R);
     __syncthreads();
-    if (t + 1 < zend) load_plane(d, u, cf, PI, t + 2, R);
+    if (t + 1 < zend) load_plane(d, u, cf, PI, t + 2, R, e);
     const float J = Jn;
     float2 b = bn;
     if (own && t + 1 < zend) {
@@ -1136,6 +1195,8 @@ __global__ void __launch_bounds__(CNT, 3) k_curv_df_residual_tiled(Dims d, CurvC
       }
       const float rv = (acc.s + acc.c) / (J * cf.h2);
       r[i] = rv;
+      if (e) u_out[i] = U(0, 0, 0);
+      if (e1) e1[i] = jacobi_value(0.f, rv, J, cf.D[i], 0.f, cf.h2, omega);
       r2 += rv * rv;
       const float fv = scale_J ? (b.x + b.y) : (b.x + b.y) / J;
       f2 += fv * fv;
@@ -1191,7 +1252,11 @@ cudaError_t launch_curv_apply(cudaStream_t st, Dims d, CurvCoef cf, const T* u, 
   return cudaGetLastError();
 }
 
-long long curv_partial_count(Dims d) {
+// the z-marching kernel copies rows in 16-byte pieces
+static bool df_march(Dims d) { return d.nx % 4 == 0 && (long long)d.nx * d.ny < (1ll << 31); }
+
+long long curv_df_partials(Dims d, int form) {
+  if (df_march(d)) return march_df_partials(d, form);
   const dim3 g = curv_tiled_grid(d);
   return (long long)g.x * g.y * g.z;
 }
@@ -1253,6 +1318,18 @@ cudaError_t launch_curv_jacobi_zero(cudaStream_t st, Dims d, const CurvCoef& cf,
   return cudaGetLastError();
 }
 
+cudaError_t launch_curv_restrict(cudaStream_t st, Dims fine, const float* f, float* rc, const CurvCoef& cc, float* e1,
+                                 float omega) {
+  const Dims dc{fine.nx / 2, fine.ny / 2, fine.nz / 2};
+  const long long cols = (long long)((dc.nx + BX - 1) / BX) * ((dc.ny + BY - 1) / BY);
+  int zc = 8;
+  while (zc > 1 && cols * ((dc.nz + zc - 1) / zc) < 4 * 152) zc /= 2;
+  k_curv_restrict<<<dim3((dc.nx + BX - 1) / BX, (dc.ny + BY - 1) / BY, (dc.nz + zc - 1) / zc), dim3(BX, BY), 0, st>>>(
+      fine, f, rc, e1, cc.J, cc.D, cc.h2, omega, zc);
+  note_launch();
+  return cudaGetLastError();
+}
+
 cudaError_t launch_curv_dense(cudaStream_t st, Dims d, CurvCoef cf, int form, double* out) {
   const long long n = ncell(d);
   k_curv_dense<<<(unsigned)((n * n + 255) / 256), 256, 0, st>>>(d, cf, form, out);
@@ -1260,11 +1337,14 @@ cudaError_t launch_curv_dense(cudaStream_t st, Dims d, CurvCoef cf, int form, do
   return cudaGetLastError();
 }
 
-cudaError_t launch_curv_df_residual(cudaStream_t st, Dims d, CurvCoef cf, const float2* src, const double* m_dev,
-                                    int scale_J, const float2* u, int form, float* r, double* pr2, double* pf2) {
+cudaError_t launch_curv_df_step(cudaStream_t st, Dims d, const CurvCoef& cf, const float2* src, const double* m_dev,
+                                int scale_J, const float2* u, const float* e, float2* u_out, int form, float* r,
+                                float* e1, float omega, double* pr2, double* pf2) {
   if (form < 0 || form > 2) return cudaErrorInvalidValue;
+  if (df_march(d))
+    return launch_march_df_step(st, d, cf, src, m_dev, scale_J, u, e, u_out, form, r, e1, omega, pr2, pf2);
   k_curv_df_residual_tiled<<<curv_tiled_grid(d), CNT, 4 * ring_slot_bytes<float2>(), st>>>(
-      d, cf, src, m_dev, scale_J, u, form, r, pr2, pf2, curv_zchunk(d));
+      d, cf, src, m_dev, scale_J, u, e, u_out, form, r, e1, omega, pr2, pf2, curv_zchunk(d));
   note_launch();
   return cudaGetLastError();
 }

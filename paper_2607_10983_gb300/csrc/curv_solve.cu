@@ -25,16 +25,10 @@ enum CurvScal { S_SUMJ = 6, S_MW = 9, S_SLAM = 10 };
 // operator form of the forward (tr false) or transposed (tr true) problem: 0 = M, 1 = M^T, 2 = S
 int curv_form(const gbmg_ctx* c, bool tr) { return c->o.curv_sym ? 2 : (tr ? 1 : 0); }
 
-// nu weighted-Jacobi sweeps; from_zero: the iterate is zero, so the first sweep is the
-// pointwise one (no read of e; the same values as a full sweep of zeros)
-gbmg_status curv_smooth(gbmg_ctx* c, int l, float*& e, float*& eo, const float* r, int nu, bool tr, bool from_zero) {
+// nu weighted-Jacobi sweeps of e (ping-pong with eo)
+gbmg_status curv_smooth(gbmg_ctx* c, int l, float*& e, float*& eo, const float* r, int nu, bool tr) {
   const Level& L = c->lv[l];
   for (int k = 0; k < nu; ++k) {
-    if (k == 0 && from_zero) {
-      TRY(launch_curv_jacobi_zero(c->stream, L.d, L.cc, r, eo, (float)c->o.omega));
-      std::swap(e, eo);
-      continue;
-    }
     ProfScope ps(c, l == 0 ? GBMG_PROF_CURV0 : GBMG_PROF_OFF);
     TRY(launch_curv_jacobi(c->stream, L.d, L.cc, r, e, eo, curv_form(c, tr), (float)c->o.omega));
     std::swap(e, eo);
@@ -43,56 +37,74 @@ gbmg_status curv_smooth(gbmg_ctx* c, int l, float*& e, float*& eo, const float* 
 }
 
 // Curvilinear V-cycle for L_l e = r (or the transposed-solve operator), one kernel
-// per operation (Sec. 4.3, Eq. curv_error; Appendix B), from e = 0: the iterate's
-// content is not read when nu1 > 0 (the first sweep is the pointwise one), and must be
-// zero otherwise.
+// per operation (Sec. 4.3, Eq. curv_error; Appendix B), from e = 0.  On entry e holds the
+// first pre-smoothing sweep, which is pointwise and written by the kernel that makes r
+// (nu1 = 0: zeros).
 gbmg_status vcycle_curv(gbmg_ctx* c, int l, float*& e, float*& eo, const float* r, bool tr) {
   const Level& L = c->lv[l];
   if (l == c->L - 1) {
     TRY(launch_coarse_matvec<float>(c->stream, c->nc, tr ? c->G32T : c->G32, r, e));
     return GBMG_OK;
   }
-  TRYS(curv_smooth(c, l, e, eo, r, c->o.nu1, tr, true));
+  TRYS(curv_smooth(c, l, e, eo, r, c->o.nu1 - 1, tr));
   TRY(launch_curv_residual(c->stream, L.d, L.cc, r, e, (float*)L.t, curv_form(c, tr)));
   const Level& C = c->lv[l + 1];
-  TRY(launch_restrict<float>(c->stream, L.d, (const float*)L.t, (float*)C.r));
   float* ce = (float*)C.e;
   float* ceo = (float*)C.e2;
-  if (l + 1 < c->L - 1 && c->o.nu1 == 0)
-    TRY(cudaMemsetAsync(ce, 0, (size_t)ncell(C.d) * sizeof(float), c->stream));
+  const bool smoothed = l + 1 < c->L - 1;
+  TRY(launch_curv_restrict(c->stream, L.d, (const float*)L.t, (float*)C.r, C.cc, smoothed && c->o.nu1 > 0 ? ce : nullptr,
+                           (float)c->o.omega));
+  if (smoothed && c->o.nu1 == 0) TRY(cudaMemsetAsync(ce, 0, (size_t)ncell(C.d) * sizeof(float), c->stream));
   TRYS(vcycle_curv(c, l + 1, ce, ceo, (const float*)C.r, tr));
   TRY(launch_prolong_add<float>(c->stream, C.d, ce, e));
-  TRYS(curv_smooth(c, l, e, eo, r, c->o.nu2, tr, false));
+  TRYS(curv_smooth(c, l, e, eo, r, c->o.nu2, tr));
+  return GBMG_OK;
+}
+
+// Buffers of one cycle: the potential before and after, and the finest level's error
+// buffer that holds the cycle's first sweep and the other one of the pair.
+struct CurvBufs {
+  float2 *phi, *phi_next;
+  float *e, *eo;
+};
+
+// The buffers after a cycle: the potential's pair swaps; the V-cycle ends in e or eo after
+// its nu1 - 1 + nu2 swaps, and the next first sweep goes to the other one.
+CurvBufs curv_next(const gbmg_ctx* c, const CurvBufs& b) {
+  const int swaps = c->L > 1 ? (c->o.nu1 > 0 ? c->o.nu1 - 1 : 0) + c->o.nu2 : 0;
+  return swaps % 2 ? CurvBufs{b.phi_next, b.phi, b.e, b.eo} : CurvBufs{b.phi_next, b.phi, b.eo, b.e};
+}
+
+// One cycle of the curvilinear solve on c->stream: FP32 V-cycle on r0, then phi_next = phi +
+// e, r0 = the double-float residual with its norm, and the next cycle's first sweep in one
+// kernel, the scalars copied to pinned host memory.  b becomes the next cycle's buffers.
+// The launches depend only on the context, the orientation and the buffers, which alternate
+// with the potential's parity, so after a cycle has run eagerly each (orientation, parity)
+// is captured once as a CUDA graph and replayed (the coefficients change in place; timed
+// families are timed by event nodes).
+gbmg_status curv_cycle(gbmg_ctx* c, bool tr, float* r0, CurvBufs& b) {
+  const Level& L0 = c->lv[0];
+  double* sc = c->scal;
+  float* e = b.e;
+  float* eo = b.eo;
+  TRYS(vcycle_curv(c, 0, e, eo, r0, tr));
+  // (a single-level hierarchy's cycle is the coarsest solve: its next cycle needs no sweep)
+  const bool first = c->L > 1 && c->o.nu1 > 0;
+  {
+    ProfScope ps(c, GBMG_PROF_DF0);
+    TRY(launch_curv_df_step(c->stream, L0.d, L0.cc, c->F_df, sc + S_MEAN_F, tr ? 0 : 1, b.phi, e, b.phi_next,
+                            curv_form(c, tr), r0, first ? eo : nullptr, (float)c->o.omega, c->partials, nullptr));
+  }
+  if (c->L > 1 && !first) TRY(cudaMemsetAsync(eo, 0, (size_t)ncell(L0.d) * sizeof(float), c->stream));
+  b = curv_next(c, b);
+  TRY(launch_finalize(c->stream, c->partials, curv_df_partials(L0.d, curv_form(c, tr)), sc + S_R2, 1.0));
+  TRY(launch_scalars_to_host(c->stream, c->scal, c->host_scal_dev, 8));
   return GBMG_OK;
 }
 
 // Mixed-precision solve of L u = f (forward, f = src - weighted mean) or of the
 // transposed problem M^T u = src - mean(src) (tr).  u_in NULL starts from zero;
-// u_out NULL leaves the result in c->phi_df only.
-// One cycle of the curvilinear solve on c->stream: FP32 V-cycle on r0, phi += e in
-// double-float, r0 = the double-float residual and its norm, the scalars copied to pinned
-// host memory.  Its launches depend only on the context and the orientation, so after a
-// cycle has run eagerly it is captured once as a CUDA graph per orientation and replayed
-// (the coefficients change in place; timed families are timed by event nodes).
-gbmg_status curv_cycle(gbmg_ctx* c, bool tr, float* r0) {
-  const Level& L0 = c->lv[0];
-  const long long n = ncell(L0.d);
-  double* sc = c->scal;
-  float* e = (float*)L0.e;
-  float* eo = (float*)L0.e2;
-  if (c->o.nu1 == 0) TRY(cudaMemsetAsync(e, 0, (size_t)n * sizeof(float), c->stream));
-  TRYS(vcycle_curv(c, 0, e, eo, r0, tr));
-  TRY(launch_df_update(c->stream, n, c->phi_df, e, nullptr));
-  {
-    ProfScope ps(c, GBMG_PROF_DF0);
-    TRY(launch_curv_df_residual(c->stream, L0.d, L0.cc, c->F_df, sc + S_MEAN_F, tr ? 0 : 1, c->phi_df, curv_form(c, tr),
-                                r0, c->partials, nullptr));
-  }
-  TRY(launch_finalize(c->stream, c->partials, curv_partial_count(L0.d), sc + S_R2, 1.0));
-  TRY(launch_scalars_to_host(c->stream, c->scal, c->host_scal_dev, 8));
-  return GBMG_OK;
-}
-
+// u_out NULL leaves the result in c->curv_phi only.
 gbmg_status curv_solve_impl(gbmg_ctx* c, const double* src, const double* u_in, double* u_out, double tol, int maxv,
                             gbmg_stats& st, bool tr) {
   const Level& L0 = c->lv[0];
@@ -101,7 +113,7 @@ gbmg_status curv_solve_impl(gbmg_ctx* c, const double* src, const double* u_in, 
   double* part1 = c->partials + c->npart;
   double* part2 = c->partials + 2 * c->npart;
   double* sc = c->scal;
-  const long long pr = df_partial_count(n), pc = curv_partial_count(L0.d);
+  const long long pr = df_partial_count(n), pc = curv_df_partials(L0.d, curv_form(c, tr));
   TRY(launch_f64_to_df(c->stream, n, src, c->F_df, part));
   if (!tr) {
     TRY(launch_wsum(c->stream, n, src, L0.cc.J, part, part1));
@@ -117,9 +129,11 @@ gbmg_status curv_solve_impl(gbmg_ctx* c, const double* src, const double* u_in, 
     TRY(cudaMemsetAsync(c->phi_df, 0, (size_t)n * sizeof(float2), c->stream));
   }
   float* r0 = (float*)L0.r;
-  const int itr = curv_form(c, tr);
-  TRY(launch_curv_df_residual(c->stream, L0.d, L0.cc, c->F_df, sc + S_MEAN_F, tr ? 0 : 1, c->phi_df, itr, r0, part,
-                              part1));
+  CurvBufs b{c->phi_df, c->phi_df2, (float*)L0.e, (float*)L0.e2};
+  const bool first = c->L > 1 && c->o.nu1 > 0;
+  TRY(launch_curv_df_step(c->stream, L0.d, L0.cc, c->F_df, sc + S_MEAN_F, tr ? 0 : 1, b.phi, nullptr, nullptr,
+                          curv_form(c, tr), r0, first ? b.e : nullptr, (float)c->o.omega, part, part1));
+  if (c->L > 1 && !first) TRY(cudaMemsetAsync(b.e, 0, (size_t)n * sizeof(float), c->stream));
   TRY(launch_finalize(c->stream, part, pc, sc + S_R2, 1.0));
   TRY(launch_finalize(c->stream, part1, pc, sc + S_F2, 1.0));
   double rel = 0.0;
@@ -130,24 +144,34 @@ gbmg_status curv_solve_impl(gbmg_ctx* c, const double* src, const double* u_in, 
   while (!mon.done()) {
     sync_graph_mask(c);
     const bool graphs = c->curv_warm[k] && !c->cyc_off;
-    if (graphs && !c->curv_exec[k])
-      TRYS(capture_graph(c, 2 + k, [&]() { return curv_cycle(c, tr, r0); }, c->curv_exec[k], c->curv_kernels[k]));
-    const bool replay = graphs && c->curv_exec[k];
+    const int g = 2 * k + (b.phi == c->phi_df ? 0 : 1);
+    CurvBufs next = b;
+    if (graphs && !c->curv_exec[g])
+      TRYS(capture_graph(c, 2 + g,
+                         [&]() {
+                           CurvBufs q = b;
+                           return curv_cycle(c, tr, r0, q);
+                         },
+                         c->curv_exec[g], c->curv_kernels[g]));
+    const bool replay = graphs && c->curv_exec[g];
     if (replay) {
-      TRY(cudaGraphLaunch(c->curv_exec[k], c->stream));
-      note_launches(c->curv_kernels[k]);
+      TRY(cudaGraphLaunch(c->curv_exec[g], c->stream));
+      note_launches(c->curv_kernels[g]);
+      next = curv_next(c, b);
     } else {
-      TRYS(curv_cycle(c, tr, r0));
+      TRYS(curv_cycle(c, tr, r0, next));
       c->curv_warm[k] = true;
     }
+    b = next;
     TRYS(rel_from_host(c, rel));
-    if (replay) gprof_collect(c, 2 + k);
+    if (replay) gprof_collect(c, 2 + g);
     if (mon.record(rel)) break;
   }
+  c->curv_phi = b.phi;
   if (u_out) {
-    TRY(launch_df_update(c->stream, n, c->phi_df, nullptr, part2));
+    TRY(launch_df_update(c->stream, n, b.phi, nullptr, part2));
     TRY(launch_finalize(c->stream, part2, pr, sc + S_MEAN_PHI, 1.0 / (double)n));
-    TRY(launch_df_to_f64(c->stream, n, c->phi_df, sc + S_MEAN_PHI, u_out));
+    TRY(launch_df_to_f64(c->stream, n, b.phi, sc + S_MEAN_PHI, u_out));
   }
   return GBMG_OK;
 }
@@ -286,18 +310,18 @@ extern "C" gbmg_status mg_solve_adjoint(gbmg_ctx* c, const double* phi_bar_dev, 
   double* sc = c->scal;
   const long long pr = df_partial_count(n);
   // lam in FP64, s_lam = sum(J lam) / sum(J), delta_bar = J (lam - s_lam)
-  TRY(launch_jscale(c->stream, n, c->phi_df, L0.cc.J, nullptr, nullptr, c->adj_lam));
+  TRY(launch_jscale(c->stream, n, c->curv_phi, L0.cc.J, nullptr, nullptr, c->adj_lam));
   TRY(launch_wsum(c->stream, n, c->adj_lam, L0.cc.J, part, part1));
   TRY(launch_finalize(c->stream, part, pr, sc + S_SUM_F, 1.0));
   TRY(launch_finalize(c->stream, part1, pr, sc + S_SUMJ, 1.0));
   TRY(launch_ratio(c->stream, sc + S_SUM_F, sc + S_SUMJ, sc + S_SLAM));
-  TRY(launch_jscale(c->stream, n, c->phi_df, L0.cc.J, sc + S_SLAM, source_bar_dev, nullptr));
+  TRY(launch_jscale(c->stream, n, c->curv_phi, L0.cc.J, sc + S_SLAM, source_bar_dev, nullptr));
   if (psi_bar_dev) {
     TRY(launch_wsum(c->stream, n, source_dev, L0.cc.J, part, part1));
     TRY(launch_finalize(c->stream, part, pr, sc + S_SUM_F, 1.0));
     TRY(launch_finalize(c->stream, part1, pr, sc + S_SUMJ, 1.0));
     TRY(launch_ratio(c->stream, sc + S_SUM_F, sc + S_SUMJ, sc + S_MW));
-    TRY(launch_psibar(c->stream, L0.d, L0.psi, phi_dev, c->phi_df, source_dev, sc + S_MW, sc + S_SLAM, L0.h,
+    TRY(launch_psibar(c->stream, L0.d, L0.psi, phi_dev, c->curv_phi, source_dev, sc + S_MW, sc + S_SLAM, L0.h,
                       c->o.curv_sym, (float2*)c->adj_S, psi_bar_dev));
   }
   TRY(cudaStreamSynchronize(c->stream));
@@ -372,7 +396,8 @@ extern "C" gbmg_status mg_curv_vcycle(gbmg_ctx* c, int transpose, const float* r
   const long long n = ncell(L0.d);
   float* e = (float*)L0.e;
   float* eo = (float*)L0.e2;
-  TRY(cudaMemsetAsync(e, 0, (size_t)n * 4, c->stream));
+  if (c->L > 1 && c->o.nu1 > 0) TRY(launch_curv_jacobi_zero(c->stream, L0.d, L0.cc, r, e, (float)c->o.omega));
+  else TRY(cudaMemsetAsync(e, 0, (size_t)n * 4, c->stream));
   TRYS(vcycle_curv(c, 0, e, eo, r, transpose != 0));
   TRY(cudaMemcpyAsync(e_out, e, (size_t)n * 4, cudaMemcpyDeviceToDevice, c->stream));
   return GBMG_OK;

@@ -179,7 +179,7 @@ extern "C" gbmg_status mg_setup(gbmg_ctx** out, int nx, int ny, int nz, int leve
   if (o.prec == GBMG_MIXED) {
     oF = take((size_t)n0 * sizeof(float2));
     oP = take((size_t)n0 * sizeof(float2));
-    if (o.fused) oP2 = take((size_t)n0 * sizeof(float2));
+    if (o.fused || curv) oP2 = take((size_t)n0 * sizeof(float2));
     oR = take((size_t)n0 * sizeof(float));
   }
   const long long np = std::max(std::max(partial_count(dims[0]), df_partial_count(n0)),
@@ -235,7 +235,7 @@ extern "C" gbmg_status mg_setup(gbmg_ctx** out, int nx, int ny, int nz, int leve
   if (o.prec == GBMG_MIXED) {
     c->F_df = (float2*)(a + oF);
     c->phi_df = (float2*)(a + oP);
-    c->phi_df2 = o.fused ? (float2*)(a + oP2) : nullptr;
+    c->phi_df2 = o.fused || curv ? (float2*)(a + oP2) : nullptr;
     c->r_alt = (float*)(a + oR);
   }
   c->npart = np;

@@ -149,11 +149,23 @@ cudaError_t launch_march_residual(cudaStream_t st, Dims d, const CurvCoef& cf, c
                                   float* out, int form);
 // dense n x n matrix of op / J on a (small) level, FP64 row-major
 cudaError_t launch_curv_dense(cudaStream_t st, Dims d, CurvCoef cf, int form, double* out);
-// double-float outer residual: r = b - op(u)/J with b = J (src - m) (scale_J) or src
-// block partial sums written by launch_curv_df_residual
-long long curv_partial_count(Dims d);
-cudaError_t launch_curv_df_residual(cudaStream_t st, Dims d, CurvCoef cf, const float2* src, const double* m_dev,
-                                    int scale_J, const float2* u, int form, float* r, double* pr2, double* pf2);
+// One double-float defect-correction step of the finest level: u_out = u + e (e NULL: no
+// update, u_out unused), r = b - op(u + e) / J with b = J (src - m) (scale_J) or src, and
+// (e1 not NULL) e1 = the first weighted-Jacobi sweep for r, from zero.
+// u, e and the coefficients are the context's own buffers (256-byte aligned); meshes with nx
+// a multiple of 4 run the z-marching kernel, others the one-cell tiles.
+long long curv_df_partials(Dims d, int form);  // block partial sums it writes
+long long march_df_partials(Dims d, int form);
+cudaError_t launch_march_df_step(cudaStream_t st, Dims d, const CurvCoef& cf, const float2* src, const double* m_dev,
+                                 int scale_J, const float2* u, const float* e, float2* u_out, int form, float* r,
+                                 float* e1, float omega, double* pr2, double* pf2);
+cudaError_t launch_curv_df_step(cudaStream_t st, Dims d, const CurvCoef& cf, const float2* src, const double* m_dev,
+                                int scale_J, const float2* u, const float* e, float2* u_out, int form, float* r,
+                                float* e1, float omega, double* pr2, double* pf2);
+// rc = full weighting of f (the finer level's field); with e1, also the first sweep for rc,
+// from zero, on the coarse level (its coefficients cc)
+cudaError_t launch_curv_restrict(cudaStream_t st, Dims fine, const float* f, float* rc, const CurvCoef& cc, float* e1,
+                                 float omega);
 // partial sums of x * J and of J (df_partial_count(n) blocks each)
 cudaError_t launch_wsum(cudaStream_t st, long long n, const double* x, const float* J, double* pxj, double* pj);
 // psi_bar of the curvilinear adjoint on the finest level from the forward solution phi

@@ -37,6 +37,9 @@ constexpr int SLOT = f_off(NF);            // floats of one ring slot
 __device__ __forceinline__ void cp_async16(unsigned dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
+__device__ __forceinline__ void cp_async8(unsigned dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
+}
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
@@ -53,14 +56,15 @@ struct Fields {
 // yz; 3 = zz.
 constexpr int f_group(int f) { return has_x(f) ? (has_y(f) ? 0 : 1) : (has_y(f) ? 2 : 3); }
 
-// The copies of one plane by NT threads (128 or 256): thread t copies chunk t of every
-// field (its place in the slot is t 16-byte units into the field); with 128 threads the
-// chunks from 128 on, of all fields one after the other, are dealt out as extras.
-template <int NT>
+// The copies of one plane of the fields F0 .. NF - 1 by NT threads (128 or 256): thread t
+// copies chunk t of every field (its place in the slot is t 16-byte units into the field);
+// with 128 threads the chunks from 128 on, of all fields one after the other, are dealt
+// out as extras.
+template <int NT, int F0 = 0>
 struct Copier {
   static constexpr int extra_count() {
     int n = 0;
-    for (int f = 0; f < NF; ++f) n += f_chunks(f) > NT ? f_chunks(f) - NT : 0;
+    for (int f = F0; f < NF; ++f) n += f_chunks(f) > NT ? f_chunks(f) - NT : 0;
     return n;
   }
   static constexpr int NE = (extra_count() + NT - 1) / NT;
@@ -85,11 +89,11 @@ struct Copier {
       x_src[k] = nullptr;
       x_dst[k] = 0;
 #pragma unroll
-      for (int f = 0; f < NF; ++f) {
+      for (int f = F0; f < NF; ++f) {
         const int n = f_chunks(f) > NT ? f_chunks(f) - NT : 0;
         if (q >= 0 && q < n) {
           x_src[k] = P.p[f] + chunk_off(d, x0, y0, has_x(f), has_y(f), NT + q);
-          x_dst[k] = (unsigned)(f_off(f) * 4 + (NT + q) * 16);
+          x_dst[k] = (unsigned)((f_off(f) - f_off(F0)) * 4 + (NT + q) * 16);
         }
         q -= n;
       }
@@ -99,9 +103,9 @@ struct Copier {
   __device__ __forceinline__ void issue(const Fields& P, long long zo, unsigned sa) const {
     const unsigned t = sa + threadIdx.x * 16u;
 #pragma unroll
-    for (int f = 0; f < NF; ++f)
+    for (int f = F0; f < NF; ++f)
       if (f_chunks(f) >= NT || threadIdx.x < f_chunks(f))
-        cp_async16(t + (unsigned)f_off(f) * 4u, P.p[f] + (zo + off[f_group(f)]));
+        cp_async16(t + (unsigned)(f_off(f) - f_off(F0)) * 4u, P.p[f] + (zo + off[f_group(f)]));
 #pragma unroll
     for (int k = 0; k < NE; ++k)
       if (x_src[k]) cp_async16(sa + x_dst[k], x_src[k] + zo);

@@ -70,7 +70,7 @@ struct gbmg_ctx {
   float* pcg = nullptr;         // conjugate-gradient vectors e, p, q (3 finest FP32 fields), first use
   float2* F_df = nullptr;       // mixed precision: source as double-float
   float2* phi_df = nullptr;     // mixed precision: potential as double-float
-  float2* phi_df2 = nullptr;    // mixed precision: second potential buffer (fused update)
+  float2* phi_df2 = nullptr;    // mixed precision: second potential buffer (fused and curvilinear updates)
   float* r_alt = nullptr;       // mixed precision: second finest residual buffer
   double* partials = nullptr;   // 4 regions of npart block partial sums
   long long npart = 0;
@@ -97,14 +97,16 @@ struct gbmg_ctx {
   cudaStream_t cap_stream = nullptr;
   bool cyc_off = false;   // a capture failed: this context launches its cycles one by one
   bool cyc_warm = false;  // a cycle has run eagerly (the kernels' one-time attributes are set)
-  // curvilinear solves: one cycle as a CUDA graph per orientation (forward, transposed)
-  cudaGraphExec_t curv_exec[2] = {nullptr, nullptr};
-  long long curv_kernels[2] = {0, 0};
+  // curvilinear solves: one cycle as a CUDA graph per orientation (forward, transposed) and
+  // parity of the potential buffers, index 2 * orientation + parity
+  cudaGraphExec_t curv_exec[4] = {};
+  long long curv_kernels[4] = {};
   bool curv_warm[2] = {false, false};
-  // kernel timing inside the cycle graphs: per graph slot (flat parity 0 / 1, curvilinear
-  // orientation 0 / 1), family and timed launch an event pair that the graph's nodes record
+  float2* curv_phi = nullptr;   // the potential buffer the last curvilinear solve ended in
+  // kernel timing inside the cycle graphs: per graph slot (flat parity 0 / 1, then the four
+  // curvilinear graphs), family and timed launch an event pair that the graph's nodes record
   // on every replay; read after each replay into the per-family totals
-  static constexpr int GSLOTS = 4, GPAIRS = 8;
+  static constexpr int GSLOTS = 6, GPAIRS = 8;
   cudaEvent_t gprof_ev[GSLOTS][8][GPAIRS][2] = {};
   int gprof_cnt[GSLOTS][8] = {};
   int cap_slot = -1;            // slot of the graph being captured (-1: none)
