@@ -3,7 +3,7 @@
 // 16^3, 8^3, 4^3).  Every cell value is computed by the per-cell functions of the
 // one-kernel-per-operation kernels in the same order, and the coarsest solve keeps
 // their warp-per-row summation order, so the result is bit-identical to that chain.
-// Used by the single-CTA kernel of small_cycle.cu and by the batched persistent kernel.
+// Used by the batched persistent kernel (single solves run the kernel of small_cycle.cu).
 #pragma once
 #include "kernels.h"
 #include "stencil.cuh"
