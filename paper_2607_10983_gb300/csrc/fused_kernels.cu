@@ -60,13 +60,25 @@ using DFT = DTile<64, 16, 2, 320>;
 
 // ---- double-float update
 
-// z chunk of the double-float update: at least four waves of two CTAs per SM, so that
-// enough loads are in flight; the warm-up costs one plane per chunk.
+// z chunk of the double-float update.  Large meshes: at least four waves of two CTAs per
+// SM, so that enough loads are in flight.  Meshes that have no four waves of 16-plane
+// chunks: the chunk with the shortest critical path, whole waves of 304 CTAs times the
+// chunk and its two extra planes (16-plane chunks left most SMs idle there: 64^3 20.2 -> 6.6
+// us, 160 x 128 x 224 42 -> 36 us, 256^3 108 -> 104 us).
 int df_zchunk(Dims d) {
   const long long tiles = (long long)((d.nx + DFT::TX - 1) / DFT::TX) * ((d.ny + DFT::TY - 1) / DFT::TY);
-  int zc = d.nz;
-  while (zc > 16 && tiles * ((d.nz + zc - 1) / zc) < 4 * 2 * 152) zc = (zc + 1) / 2;
-  return zc;
+  if (tiles * ((d.nz + 15) / 16) >= 4 * 2 * 152) {
+    int zc = d.nz;
+    while (tiles * ((d.nz + zc - 1) / zc) < 4 * 2 * 152) zc = (zc + 1) / 2;
+    return zc;
+  }
+  int best = d.nz;
+  long long best_cost = -1;
+  for (int zc = 2; zc <= d.nz; ++zc) {
+    const long long waves = (tiles * ((d.nz + zc - 1) / zc) + 2 * 152 - 1) / (2 * 152);
+    if (best_cost < 0 || waves * (zc + 2) < best_cost) best_cost = waves * (zc + 2), best = zc;
+  }
+  return best;
 }
 
 long long df_update_residual_partials(Dims d) {
