@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "kernels.h"
+#include "loop.h"
 #include "solver.h"
 
 using namespace gbmg;
@@ -76,13 +77,14 @@ CurvBufs curv_next(const gbmg_ctx* c, const CurvBufs& b) {
 }
 
 // One cycle of the curvilinear solve on c->stream: FP32 V-cycle on r0, then phi_next = phi +
-// e, r0 = the double-float residual with its norm, and the next cycle's first sweep in one
-// kernel, the scalars copied to pinned host memory.  b becomes the next cycle's buffers.
-// The launches depend only on the context, the orientation and the buffers, which alternate
+// e, r0 = the double-float residual with the partial sums of its norm, and the next cycle's
+// first sweep in one kernel.  b becomes the next cycle's buffers.  curv_cycle adds the norm
+// and copies the scalars to pinned host memory.  Without timed families the whole loop is
+// one graph (loop.h); otherwise: the launches depend only on the context, the orientation and the buffers, which alternate
 // with the potential's parity, so after a cycle has run eagerly each (orientation, parity)
 // is captured once as a CUDA graph and replayed (the coefficients change in place; timed
 // families are timed by event nodes).
-gbmg_status curv_cycle(gbmg_ctx* c, bool tr, float* r0, CurvBufs& b) {
+gbmg_status curv_cycle_step(gbmg_ctx* c, bool tr, float* r0, CurvBufs& b) {
   const Level& L0 = c->lv[0];
   double* sc = c->scal;
   float* e = b.e;
@@ -97,6 +99,12 @@ gbmg_status curv_cycle(gbmg_ctx* c, bool tr, float* r0, CurvBufs& b) {
   }
   if (c->L > 1 && !first) TRY(cudaMemsetAsync(eo, 0, (size_t)ncell(L0.d) * sizeof(float), c->stream));
   b = curv_next(c, b);
+  return GBMG_OK;
+}
+gbmg_status curv_cycle(gbmg_ctx* c, bool tr, float* r0, CurvBufs& b) {
+  const Level& L0 = c->lv[0];
+  double* sc = c->scal;
+  TRYS(curv_cycle_step(c, tr, r0, b));
   TRY(launch_finalize(c->stream, c->partials, curv_df_partials(L0.d, curv_form(c, tr)), sc + S_R2, 1.0));
   TRY(launch_scalars_to_host(c->stream, c->scal, c->host_scal_dev, 8));
   return GBMG_OK;
@@ -134,13 +142,30 @@ gbmg_status curv_solve_impl(gbmg_ctx* c, const double* src, const double* u_in, 
   TRY(launch_curv_df_step(c->stream, L0.d, L0.cc, c->F_df, sc + S_MEAN_F, tr ? 0 : 1, b.phi, nullptr, nullptr,
                           curv_form(c, tr), r0, first ? b.e : nullptr, (float)c->o.omega, part, part1));
   if (c->L > 1 && !first) TRY(cudaMemsetAsync(b.e, 0, (size_t)n * sizeof(float), c->stream));
+  const int k = tr ? 1 : 0;
+  if (loop_usable(c) && !c->loop_exec[k]) {
+    CurvBufs q = b;
+    build_loop(c, [&]() { return curv_cycle_step(c, tr, r0, q); }, pc, c->loop_exec[k], c->loop_kernels[k]);
+  }
+  if (loop_usable(c) && c->loop_exec[k]) {
+    TRY(launch_loop_begin(c->stream, part, part1, pc, tol, maxv, sc + S_R2, sc + S_F2, c->loop_dev, c->loop_host_dev));
+    TRYS(loop_launch(c, c->loop_exec[k]));
+    if (u_out) {
+      const int* cycles = &c->loop_dev->cycles;
+      TRY(launch_df_update(c->stream, n, c->phi_df, nullptr, part2, c->phi_df2, cycles));
+      TRY(launch_finalize(c->stream, part2, pr, sc + S_MEAN_PHI, 1.0 / (double)n));
+      TRY(launch_df_to_f64(c->stream, n, c->phi_df, sc + S_MEAN_PHI, u_out, c->phi_df2, cycles));
+    }
+    TRYS(loop_result(c, c->loop_kernels[k], st));
+    c->curv_phi = st.cycles % 2 ? c->phi_df2 : c->phi_df;
+    return GBMG_OK;
+  }
   TRY(launch_finalize(c->stream, part, pc, sc + S_R2, 1.0));
   TRY(launch_finalize(c->stream, part1, pc, sc + S_F2, 1.0));
   double rel = 0.0;
   TRYS(read_rel(c, rel));
   Monitor mon(st, tol, maxv);
   mon.start(rel);
-  const int k = tr ? 1 : 0;
   while (!mon.done()) {
     sync_graph_mask(c);
     const bool graphs = c->curv_warm[k] && !c->cyc_off;

@@ -299,8 +299,15 @@ __global__ void k_f64_to_df_x2(long long n, const double2* __restrict__ x, float
   }
 }
 
-__global__ void k_df_to_f64_x2(long long n, const float4* __restrict__ in, const double* __restrict__ shift,
-                               double2* __restrict__ out) {
+// the input of the kernels after a device-side loop: b after an odd count of cycles
+template <typename V>
+__device__ __forceinline__ const V* by_parity(const V* a, const V* b, const int* cycles) {
+  return cycles && (*cycles & 1) ? b : a;
+}
+
+__global__ void k_df_to_f64_x2(long long n, const float4* in_a, const float4* in_b, const int* __restrict__ cycles,
+                               const double* __restrict__ shift, double2* __restrict__ out) {
+  const float4* __restrict__ in = by_parity(in_a, in_b, cycles);
   float2 ms = make_float2(0.f, 0.f);
   if (shift) {
     ms = f64_to_df(shift[0]);
@@ -332,8 +339,9 @@ __global__ void k_df_to_f64_x2(long long n, const float4* __restrict__ in, const
   }
 }
 
-__global__ void k_df_to_f64(long long n, const float2* __restrict__ in, const double* __restrict__ shift,
-                            double* __restrict__ out) {
+__global__ void k_df_to_f64(long long n, const float2* in_a, const float2* in_b, const int* __restrict__ cycles,
+                            const double* __restrict__ shift, double* __restrict__ out) {
+  const float2* __restrict__ in = by_parity(in_a, in_b, cycles);
   float2 ms = make_float2(0.f, 0.f);
   if (shift) {
     ms = f64_to_df(shift[0]);
@@ -372,9 +380,10 @@ __global__ void k_df_residual(Dims d, const float2* __restrict__ F, const double
   }
 }
 
-__global__ void k_df_update(long long n, float2* __restrict__ phi, const float* __restrict__ e,
-                            double* __restrict__ ps) {
+__global__ void k_df_update(long long n, float2* phi_a, float2* phi_b, const int* __restrict__ cycles,
+                            const float* __restrict__ e, double* __restrict__ ps) {
   __shared__ double sh[32];
+  float2* __restrict__ phi = const_cast<float2*>(by_parity(phi_a, phi_b, cycles));
   DfAcc s{0.f, 0.f};
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     float2 v = phi[i];
@@ -496,12 +505,15 @@ cudaError_t launch_f64_to_df(cudaStream_t st, long long n, const double* x, floa
   note_launch();
   return cudaGetLastError();
 }
-cudaError_t launch_df_to_f64(cudaStream_t st, long long n, const float2* in, const double* shift, double* out) {
-  if (aligned16(in, out))
-    k_df_to_f64_x2<<<red_blocks(n), RED_THREADS, 0, st>>>(n, reinterpret_cast<const float4*>(in), shift,
+cudaError_t launch_df_to_f64(cudaStream_t st, long long n, const float2* in, const double* shift, double* out,
+                             const float2* in_odd, const int* cycles) {
+  if (!cycles) in_odd = in;
+  if (aligned16(in, out) && aligned16(in_odd, out))
+    k_df_to_f64_x2<<<red_blocks(n), RED_THREADS, 0, st>>>(n, reinterpret_cast<const float4*>(in),
+                                                           reinterpret_cast<const float4*>(in_odd), cycles, shift,
                                                            reinterpret_cast<double2*>(out));
   else
-    k_df_to_f64<<<red_blocks(n), RED_THREADS, 0, st>>>(n, in, shift, out);
+    k_df_to_f64<<<red_blocks(n), RED_THREADS, 0, st>>>(n, in, in_odd, cycles, shift, out);
   note_launch();
   return cudaGetLastError();
 }
@@ -511,8 +523,9 @@ cudaError_t launch_df_residual(cudaStream_t st, Dims d, const float2* F, const d
   note_launch();
   return cudaGetLastError();
 }
-cudaError_t launch_df_update(cudaStream_t st, long long n, float2* phi, const float* e, double* ps) {
-  k_df_update<<<red_blocks(n), RED_THREADS, 0, st>>>(n, phi, e, ps);
+cudaError_t launch_df_update(cudaStream_t st, long long n, float2* phi, const float* e, double* ps, float2* phi_odd,
+                             const int* cycles) {
+  k_df_update<<<red_blocks(n), RED_THREADS, 0, st>>>(n, phi, phi_odd, cycles, e, ps);
   note_launch();
   return cudaGetLastError();
 }

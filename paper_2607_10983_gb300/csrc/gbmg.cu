@@ -47,6 +47,9 @@ gbmg_ctx::~gbmg_ctx() {
       for (auto& pr : fam)
         for (cudaEvent_t ev : pr)
           if (ev) cudaEventDestroy(ev);
+  for (cudaGraphExec_t g : loop_exec)
+    if (g) cudaGraphExecDestroy(g);
+  if (loop_ev) cudaEventDestroy(loop_ev);
   if (cap_stream) cudaStreamDestroy(cap_stream);
   for (auto& v : prof_ev)
     for (cudaEvent_t e : v) cudaEventDestroy(e);
@@ -186,6 +189,7 @@ extern "C" gbmg_status mg_setup(gbmg_ctx** out, int nx, int ny, int nz, int leve
                                 df_update_residual_partials(dims[0]));
   const size_t oPart = take((size_t)np * 4 * sizeof(double));
   const size_t oScal = take(64 * sizeof(double));
+  const size_t oLoop = take(sizeof(LoopState));
   const size_t oG64 = take((size_t)nc * nc * sizeof(double));
   const size_t oG32 = take((size_t)nc * nc * sizeof(float));
   size_t oG64T = 0, oG32T = 0, oDense = 0;
@@ -200,12 +204,14 @@ extern "C" gbmg_status mg_setup(gbmg_ctx** out, int nx, int ny, int nz, int leve
     delete c;
     return cuda_fail(e, "mg_setup: workspace allocation");
   }
-  e = cudaMallocHost((void**)&c->host_scal, 64 * sizeof(double));
+  e = cudaMallocHost((void**)&c->host_scal, 64 * sizeof(double) + sizeof(LoopState));
   if (e == cudaSuccess) e = cudaHostGetDevicePointer((void**)&c->host_scal_dev, c->host_scal, 0);
   if (e != cudaSuccess) {
     delete c;
     return cuda_fail(e, "mg_setup: pinned allocation");
   }
+  c->loop_host = (LoopState*)(c->host_scal + 64);
+  c->loop_host_dev = (LoopState*)(c->host_scal_dev + 64);
   char* a = c->arena;
   c->lv.resize(dims.size());
   for (size_t l = 0; l < dims.size(); ++l) {
@@ -241,6 +247,7 @@ extern "C" gbmg_status mg_setup(gbmg_ctx** out, int nx, int ny, int nz, int leve
   c->npart = np;
   c->partials = (double*)(a + oPart);
   c->scal = (double*)(a + oScal);
+  c->loop_dev = (LoopState*)(a + oLoop);
   c->G64 = (double*)(a + oG64);
   c->G32 = (float*)(a + oG32);
 
@@ -289,6 +296,7 @@ extern "C" gbmg_status mg_set_cycle_graphs(gbmg_ctx* ctx, int enable) {
   cudaError_t e = cudaStreamSynchronize(ctx->stream);
   if (e != cudaSuccess) return cuda_fail(e, "mg_set_cycle_graphs");
   ctx->cyc_off = enable == 0;
+  if (enable) ctx->loop_off = false;
   ctx->graph_mask = -1;  // drop the graphs captured so far
   sync_graph_mask(ctx);
   return GBMG_OK;

@@ -76,14 +76,16 @@ cudaError_t launch_scalars_to_host(cudaStream_t st, const double* src, double* d
 // ---- double-float path (finest level, h = 1) ----
 cudaError_t launch_f64_to_df(cudaStream_t st, long long n, const double* x, float2* out,
                              double* partials_sum);
+// cycles (nullable, with in_odd): a device count; in_odd is read instead when it is odd
 cudaError_t launch_df_to_f64(cudaStream_t st, long long n, const float2* in, const double* shift_dev,
-                             double* out);
+                             double* out, const float2* in_odd = nullptr, const int* cycles = nullptr);
 cudaError_t launch_df_residual(cudaStream_t st, Dims d, const float2* F, const double* m_dev,
                                const float2* phi, float* r, double* partials_r2,
                                double* partials_f2);
 // phi += e (e NULL: phi unchanged); partials_sum (nullable) gets the block sums of phi.
-cudaError_t launch_df_update(cudaStream_t st, long long n, float2* phi, const float* e,
-                             double* partials_sum);
+// phi_odd, cycles as above.
+cudaError_t launch_df_update(cudaStream_t st, long long n, float2* phi, const float* e, double* partials_sum,
+                             float2* phi_odd = nullptr, const int* cycles = nullptr);
 long long df_partial_count(long long n);
 
 // ---- conjugate-gradient vectors (FP32, device scalars): partials of a . b

@@ -5,6 +5,7 @@
 #include <vector>
 
 #include "kernels.h"
+#include "loop.h"
 #include "solver.h"
 
 using namespace gbmg;
@@ -169,6 +170,14 @@ gbmg_status vcycle_fused(gbmg_ctx* c, int l, float*& e, const float* r) {
 // Device scalar slots of the conjugate-gradient correction.
 enum PcgScal { S_RZ = 16, S_RZ_NEW = 17, S_PQ = 18 };
 
+// The conjugate-gradient vectors, allocated on first use.
+gbmg_status pcg_vectors(gbmg_ctx* c) {
+  if (c->pcg) return GBMG_OK;
+  TRY(cudaMalloc((void**)&c->pcg, (size_t)ncell(c->lv[0].d) * 3 * sizeof(float)));
+  c->owned.push_back(c->pcg);
+  return GBMG_OK;
+}
+
 // k = c->o.krylov steps of conjugate gradients for the finest FP32 error equation
 // A e = r, preconditioned by one V-cycle from zero (Sec. 3.2).  A and the V-cycle are
 // both negative definite on zero-mean fields, so these are the iterates of CG on -A
@@ -177,10 +186,7 @@ enum PcgScal { S_RZ = 16, S_RZ_NEW = 17, S_PQ = 18 };
 gbmg_status pcg_correction(gbmg_ctx* c, float* r, float*& e_out) {
   const Level& L0 = c->lv[0];
   const long long n = ncell(L0.d);
-  if (!c->pcg) {
-    TRY(cudaMalloc((void**)&c->pcg, (size_t)n * 3 * sizeof(float)));
-    c->owned.push_back(c->pcg);
-  }
+  TRYS(pcg_vectors(c));
   float* E = c->pcg;
   float* P = c->pcg + n;
   float* Q = c->pcg + 2 * n;
@@ -229,14 +235,43 @@ gbmg_status solve_fp64(gbmg_ctx* c, const double* F, double* phi, double tol, in
   TRY(launch_finalize(c->stream, part, pr, sc + S_MEAN_F, 1.0 / (double)n));
   double* f0 = (double*)L0.r;
   TRY(launch_shift<double>(c->stream, n, F, sc + S_MEAN_F, f0));
-  TRY(launch_sum<double>(c->stream, n, f0, nullptr, part));
-  TRY(launch_finalize(c->stream, part, pr, sc + S_F2, 1.0));
   double* u = (double*)L0.e;
   double* uo = (double*)L0.e2;
   TRY(cudaMemcpyAsync(u, phi, (size_t)n * sizeof(double), cudaMemcpyDeviceToDevice, c->stream));
+  const long long pc = partial_count(L0.d);
+  auto residual = [&](double* p) -> gbmg_status {
+    TRY(launch_residual<double>(c->stream, L0.d, f0, u, (double*)L0.t, 1.0, p));
+    return GBMG_OK;
+  };
+  // the sweeps of a cycle bring u back to its buffer (always with the Chebyshev smoother):
+  // the whole loop as one graph
+  const bool home = c->o.smoother == GBMG_SMOOTH_CHEBYSHEV || (c->o.nu1 + c->o.nu2) % 2 == 0;
+  if (home && loop_usable(c) && !c->loop_exec[0])
+    build_loop(c,
+               [&]() -> gbmg_status {
+                 TRYS(vcycle_unfused<double>(c, 0, u, uo, f0));
+                 return residual(part);
+               },
+               pc, c->loop_exec[0], c->loop_kernels[0]);
+  if (home && loop_usable(c) && c->loop_exec[0]) {
+    double* part1 = c->partials + c->npart;
+    TRY(launch_sum<double>(c->stream, n, f0, nullptr, part1));
+    if (pr < pc) TRY(cudaMemsetAsync(part1 + pr, 0, (size_t)(pc - pr) * sizeof(double), c->stream));
+    TRYS(residual(part));
+    if (pc < pr) TRY(cudaMemsetAsync(part + pc, 0, (size_t)(pr - pc) * sizeof(double), c->stream));
+    TRY(launch_loop_begin(c->stream, part, part1, std::max(pr, pc), tol, maxv, sc + S_R2, sc + S_F2, c->loop_dev,
+                          c->loop_host_dev));
+    TRYS(loop_launch(c, c->loop_exec[0]));
+    TRY(launch_sum<double>(c->stream, n, u, part, nullptr));
+    TRY(launch_finalize(c->stream, part, pr, sc + S_MEAN_PHI, 1.0 / (double)n));
+    TRY(launch_shift<double>(c->stream, n, u, sc + S_MEAN_PHI, phi));
+    return loop_result(c, c->loop_kernels[0], st);
+  }
+  TRY(launch_sum<double>(c->stream, n, f0, nullptr, part));
+  TRY(launch_finalize(c->stream, part, pr, sc + S_F2, 1.0));
   auto resnorm = [&]() -> gbmg_status {
-    TRY(launch_residual<double>(c->stream, L0.d, f0, u, (double*)L0.t, 1.0, part));
-    TRY(launch_finalize(c->stream, part, partial_count(L0.d), sc + S_R2, 1.0));
+    TRYS(residual(part));
+    TRY(launch_finalize(c->stream, part, pc, sc + S_R2, 1.0));
     return GBMG_OK;
   };
   TRYS(resnorm());
@@ -258,9 +293,8 @@ gbmg_status solve_fp64(gbmg_ctx* c, const double* F, double* phi, double tol, in
 
 // One cycle of the fused mixed solve on c->stream: the correction e of r0 (a V-cycle from
 // zero, or the preconditioned CG steps of krylov, which overwrite r0), phi_nxt = phi_cur +
-// e and r_nxt = F - m - A phi_nxt in double-float with their norms, and the scalars copied
-// to pinned host memory (read after the stream is synchronised).
-gbmg_status fused_cycle(gbmg_ctx* c, const float2* phi_cur, float2* phi_nxt, float* r0, float* r_nxt) {
+// e and r_nxt = F - m - A phi_nxt in double-float with the partial sums of their norms.
+gbmg_status fused_cycle_step(gbmg_ctx* c, const float2* phi_cur, float2* phi_nxt, float* r0, float* r_nxt) {
   const Level& L0 = c->lv[0];
   double* sc = c->scal;
   double* part = c->partials;
@@ -273,12 +307,19 @@ gbmg_status fused_cycle(gbmg_ctx* c, const float2* phi_cur, float2* phi_nxt, flo
     TRY(launch_df_update_residual(c->stream, L0.d, phi_cur, e, c->F_df, sc + S_MEAN_F, phi_nxt, r_nxt, part, part2,
                                   nullptr));
   }
-  TRY(launch_finalize(c->stream, part, df_update_residual_partials(L0.d), sc + S_R2, 1.0));
+  return GBMG_OK;
+}
+// The same with the norm and the scalars copied to pinned host memory (read after the
+// stream is synchronised).
+gbmg_status fused_cycle(gbmg_ctx* c, const float2* phi_cur, float2* phi_nxt, float* r0, float* r_nxt) {
+  TRYS(fused_cycle_step(c, phi_cur, phi_nxt, r0, r_nxt));
+  TRY(launch_finalize(c->stream, c->partials, df_update_residual_partials(c->lv[0].d), c->scal + S_R2, 1.0));
   TRY(launch_scalars_to_host(c->stream, c->scal, c->host_scal_dev, 8));
   return GBMG_OK;
 }
 
-// Cycles run as CUDA graphs (on small meshes the kernels are short, so launching them
+// Without timed families the whole loop is one graph (loop.h).  Otherwise cycles run as CUDA
+// graphs (on small meshes the kernels are short, so launching them
 // one by one from the host would leave the GPU waiting; on large ones the host is ahead
 // except right after each cycle's convergence check): one graph per parity of the
 // potential buffers, captured the first time that parity comes up after a cycle of the
@@ -307,6 +348,27 @@ gbmg_status solve_mixed(gbmg_ctx* c, const double* F, const double* phi, double*
   if (c->o.fused) {
     TRY(launch_df_update_residual(c->stream, L0.d, c->phi_df, nullptr, c->F_df, sc + S_MEAN_F, nullptr, r0, part,
                                   part2, part1));
+    if (loop_usable(c) && !c->loop_exec[0]) {
+      if (c->o.krylov) TRYS(pcg_vectors(c));  // (not during the capture)
+      float2 *pa = c->phi_df, *pb = c->phi_df2;
+      float *ra = r0, *rb = c->r_alt;
+      build_loop(c,
+                 [&]() -> gbmg_status {
+                   TRYS(fused_cycle_step(c, pa, pb, ra, rb));
+                   std::swap(pa, pb);
+                   std::swap(ra, rb);
+                   return GBMG_OK;
+                 },
+                 pu, c->loop_exec[0], c->loop_kernels[0]);
+    }
+    if (loop_usable(c) && c->loop_exec[0]) {
+      TRY(launch_loop_begin(c->stream, part, part1, pu, tol, maxv, sc + S_R2, sc + S_F2, c->loop_dev, c->loop_host_dev));
+      TRYS(loop_launch(c, c->loop_exec[0]));
+      // epilogue: gauge and conversion of the buffer the last cycle wrote
+      TRY(launch_finalize(c->stream, part2, pu, sc + S_MEAN_PHI, 1.0 / (double)n));
+      TRY(launch_df_to_f64(c->stream, n, c->phi_df, sc + S_MEAN_PHI, phi_out, c->phi_df2, &c->loop_dev->cycles));
+      return loop_result(c, c->loop_kernels[0], st);
+    }
     TRY(launch_finalize(c->stream, part, pu, sc + S_R2, 1.0));
     TRY(launch_finalize(c->stream, part1, pu, sc + S_F2, 1.0));
   } else {

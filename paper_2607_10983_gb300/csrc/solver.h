@@ -33,6 +33,13 @@ gbmg_status curv_solve(gbmg_ctx* c, const double* F, double* phi, double tol, in
 // Parameters of the single-CTA bottom cycle from level l (false when it does not apply).
 bool small_cycle_params(const gbmg_ctx* c, int l, SmallCycle* out);
 
+// Books of a solve's device-side cycle loop (Monitor of host_math.h on the device).
+struct LoopState {
+  int cycles, maxv, status, go;
+  double tol, f2, rel0, rel, prev1, prev2;
+  double hist[64];
+};
+
 // Slots of the device scalar area gbmg_ctx::scal.
 enum Scal {
   S_SUM_F = 0,   // sum of F, then its mean
@@ -103,6 +110,14 @@ struct gbmg_ctx {
   long long curv_kernels[4] = {};
   bool curv_warm[2] = {false, false};
   float2* curv_phi = nullptr;   // the potential buffer the last curvilinear solve ended in
+  // the whole loop of a solve as one graph (loop.h): flat or forward curvilinear, transposed
+  cudaGraphExec_t loop_exec[2] = {nullptr, nullptr};
+  long long loop_kernels[2] = {0, 0};
+  bool loop_off = false;  // building a loop failed: a graph launch per cycle instead
+  gbmg::LoopState* loop_dev = nullptr;
+  gbmg::LoopState* loop_host = nullptr;      // mapped host copy of the books
+  gbmg::LoopState* loop_host_dev = nullptr;  // its device address
+  cudaEvent_t loop_ev = nullptr;
   // kernel timing inside the cycle graphs: per graph slot (flat parity 0 / 1, then the four
   // curvilinear graphs), family and timed launch an event pair that the graph's nodes record
   // on every replay; read after each replay into the per-family totals

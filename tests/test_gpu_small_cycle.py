@@ -9,7 +9,7 @@ torch = pytest.importorskip("torch")
 
 
 @pytest.mark.parametrize("degree", [1, 3, 4])
-@pytest.mark.parametrize("shape", [(16, 16, 16), (20, 40, 40), (10, 20, 20), (28, 20, 12), (8, 8, 64), (12, 24, 8),
+@pytest.mark.parametrize("shape", [(16, 16, 16), (20, 40, 40), (10, 20, 20), (8, 20, 24), (8, 8, 64), (12, 24, 8),
                                    (64, 64, 64), (14, 10, 10)])
 def test_small_cycle_equals_chain(gb, shape, degree):
     r = torch.randn(shape, generator=torch.Generator(device="cuda").manual_seed(91), device="cuda")
