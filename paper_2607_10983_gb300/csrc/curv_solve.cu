@@ -11,7 +11,6 @@
 // delta_bar = J (lam - sum(J lam)/sum(J)), psi_bar through the geometry.
 // With the symmetric variant (opts.curv_sym) both solves use S, its own transpose.
 #include <cstring>
-#include <vector>
 
 #include "kernels.h"
 #include "loop.h"
@@ -21,7 +20,7 @@ using namespace gbmg;
 
 namespace {
 
-enum CurvScal { S_SUMJ = 6, S_MW = 9, S_SLAM = 10 };
+enum CurvScal { S_SUMJ = 6, S_MW = 9, S_SLAM = 10, S_PINV = 20 };  // (S_PINV holds an int)
 
 // operator form of the forward (tr false) or transposed (tr true) problem: 0 = M, 1 = M^T, 2 = S
 int curv_form(const gbmg_ctx* c, bool tr) { return c->o.curv_sym ? 2 : (tr ? 1 : 0); }
@@ -236,21 +235,19 @@ gbmg_status build_diag(gbmg_ctx* c) {
 gbmg_status build_coarsest(gbmg_ctx* c, const char* who) {
   const Level& C = c->lv[c->L - 1];
   const int nc = c->nc;
-  std::vector<float> Jc(nc);
-  TRY(cudaMemcpyAsync(Jc.data(), C.cc.J, (size_t)nc * sizeof(float), cudaMemcpyDeviceToHost, c->stream));
-  std::vector<double> Lm((size_t)nc * nc), G;
-  for (int tr = 0; tr < 2; ++tr) {
-    TRY(launch_curv_dense(c->stream, C.d, C.cc, curv_form(c, tr != 0), c->dense));
-    TRY(cudaMemcpyAsync(Lm.data(), c->dense, Lm.size() * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    TRY(cudaStreamSynchronize(c->stream));
-    std::vector<double> w(Jc.begin(), Jc.end());
-    for (float v : Jc)
-      if (!(v > 0.f)) return fail(GBMG_ERR_INVALID_ARG, std::string(who) + ": non-positive volume element on the coarsest level");
-    if (!dense_pinv(nc, Lm, w, G)) return fail(GBMG_ERR_INVALID_ARG, std::string(who) + ": coarsest operator is singular");
-    std::vector<float> G32(G.begin(), G.end());
-    TRY(cudaMemcpy(tr ? c->G64T : c->G64, G.data(), G.size() * sizeof(double), cudaMemcpyHostToDevice));
-    TRY(cudaMemcpy(tr ? c->G32T : c->G32, G32.data(), G32.size() * sizeof(float), cudaMemcpyHostToDevice));
-  }
+  const size_t n2 = (size_t)nc * nc;
+  int* const status = reinterpret_cast<int*>(c->scal + S_PINV);
+  for (int tr = 0; tr < 2; ++tr)
+    TRY(launch_curv_dense(c->stream, C.d, C.cc, curv_form(c, tr != 0), c->dense + tr * n2));
+  TRY(launch_coarse_inverse(c->stream, nc, c->dense, c->dense + 2 * n2, C.cc.J, c->G64, c->G64T, c->G32, c->G32T,
+                            status));
+  TRY(launch_scalars_to_host(c->stream, c->scal + S_PINV, c->host_scal_dev + S_PINV, 1));
+  TRY(cudaStreamSynchronize(c->stream));
+  int flags;
+  std::memcpy(&flags, c->host_scal + S_PINV, sizeof(flags));
+  if (flags & 4) return fail(GBMG_ERR_CUDA, std::string(who) + ": the coarsest inversion timed out");
+  if (flags & 2) return fail(GBMG_ERR_INVALID_ARG, std::string(who) + ": non-positive volume element on the coarsest level");
+  if (flags & 1) return fail(GBMG_ERR_INVALID_ARG, std::string(who) + ": coarsest operator is singular");
   return GBMG_OK;
 }
 

@@ -196,7 +196,8 @@ extern "C" gbmg_status mg_setup(gbmg_ctx** out, int nx, int ny, int nz, int leve
   if (curv) {
     oG64T = take((size_t)nc * nc * sizeof(double));
     oG32T = take((size_t)nc * nc * sizeof(float));
-    oDense = take((size_t)nc * nc * sizeof(double));
+    // the two dense operators and the scratch of their inversion
+    oDense = take((size_t)nc * nc * 2 * sizeof(double) + coarse_inverse_work((int)nc));
   }
   c->arena_bytes = off;
   e = cudaMalloc((void**)&c->arena, off);

@@ -151,6 +151,13 @@ cudaError_t launch_march_residual(cudaStream_t st, Dims d, const CurvCoef& cf, c
                                   float* out, int form);
 // dense n x n matrix of op / J on a (small) level, FP64 row-major
 cudaError_t launch_curv_dense(cudaStream_t st, Dims d, CurvCoef cf, int form, double* out);
+// Minimum-norm inverses (dense_pinv) of two dense n x n FP64 operators (the coarsest
+// operator and its transposed-solve twin, dense) with left null vector J, n <= 512, in FP64
+// and FP32; work: coarse_inverse_work(n) bytes.  status (device): bit 0 a singular operator,
+// bit 1 a J that is not positive, bit 2 a bounded wait inside the kernel ran out.
+size_t coarse_inverse_work(int n);
+cudaError_t launch_coarse_inverse(cudaStream_t st, int n, const double* dense, void* work, const float* J,
+                                  double* g64, double* g64t, float* g32, float* g32t, int* status);
 // One double-float defect-correction step of the finest level: u_out = u + e (e NULL: no
 // update, u_out unused), r = b - op(u + e) / J with b = J (src - m) (scale_J) or src, and
 // (e1 not NULL) e1 = the first weighted-Jacobi sweep for r, from zero.

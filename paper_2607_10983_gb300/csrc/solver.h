@@ -66,7 +66,7 @@ struct gbmg_ctx {
   float* G32 = nullptr;
   double* G64T = nullptr;       // curvilinear: pseudo-inverse of the transposed-solve operator
   float* G32T = nullptr;
-  double* dense = nullptr;      // curvilinear: nc x nc scratch for the coarsest operator
+  double* dense = nullptr;      // curvilinear: scratch of the coarsest inverses (launch_coarse_inverse)
   bool geom_ready = false;      // curvilinear: mg_set_geometry or mg_set_coefficients has run
   bool geom_from_psi = false;   // the coefficients were built from psi (psi_bar needs psi)
   bool fused_all = false;       // testing: blocked kernels on every level of at least 16^3
