@@ -260,7 +260,7 @@ gbmg_status mg_cic_read(gbmg_ctx* ctx, const double* field_dev, int ncomp, const
 /* Single-precision force at the particles (the paper's PM force evaluation runs in FP32):
  * phi (FP64) rounded to FP32, force grid -grad4 phi (the fourth-order gradient of mg_grad,
  * h = 1) in FP32, then CIC read in FP32 with the weights of mg_cic_paint.
- * force_out_dev: n_particles x 3 FP32 (x, y, z).  Allocates 16 bytes per cell of scratch on
+ * force_out_dev: n_particles x 3 FP32 (x, y, z).  Allocates 20 bytes per cell of scratch on
  * first use (kept until mg_destroy).  Queued on the context's stream. */
 gbmg_status mg_force(gbmg_ctx* ctx, const double* phi_dev, const float* pos_dev, long long n_particles,
                      float* force_out_dev);
