@@ -298,7 +298,9 @@ gbmg_status mg_batch_set_tiles(gbmg_batch* batch, const int* tile_cells, int nle
 gbmg_status mg_batch_get_tiles(const gbmg_batch* batch, int* tile_cells, int nlevels);
 /* on != 0: run each solve as a CUDA graph (captured at the first solve on a stream of
  * the batch's own, replayed while tol, max_vcycles, grid and tile sizes are unchanged;
- * ordered after earlier and before later work on the batch's stream).  Off by default. */
+ * ordered after earlier and before later work on the batch's stream).  Where every problem
+ * has a bottom cycle (degrees 1 to 4) the graph runs the phases as kernels of their own
+ * in a loop on the device, otherwise the persistent kernel.  Off by default. */
 gbmg_status mg_batch_use_graph(gbmg_batch* batch, int on);
 /* Number of levels of the deepest problem (length of the tile-size array). */
 int mg_batch_num_levels(const gbmg_batch* batch);

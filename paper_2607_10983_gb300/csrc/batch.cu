@@ -23,22 +23,16 @@
 #include <cstring>
 #include <vector>
 
-#include "dfk.cuh"
-#include "kernels.h"
-#include "legs.cuh"
+#include "batch.cuh"
 #include "small_cycle.cuh"
-#include "solver.h"
-#include "stencil.cuh"
 
 namespace cg = cooperative_groups;
 using namespace gbmg;
 
 namespace {
 
-constexpr int BMAXL = 16;
-constexpr int CHUNK = 4096;      // default tile (chunk) size in cells
-constexpr int MINCHUNK = 1024;   // smallest tile the tables are sized for
-constexpr int MAXCHUNK = 65536;
+using namespace batchk;
+
 constexpr int BT = 384;          // block size (the fused legs' thread-column layout)
 constexpr int DFZC = 32;         // z planes per item of the fused double-float phase
 
@@ -59,75 +53,6 @@ struct BUp {
 // double-float items: 32 x 32 tiles, which 64^3, 96^3 and 128^3 meshes fill whole (64 x 16
 // tiles left half of every second tile column empty on 96^3; measured 3095 -> 3132 solves/s)
 using BDf = dfk::DTile<32, 32, 2, BT>;
-
-// per-problem scalars
-enum { P_MEAN = 0, P_F2 = 1, P_R2 = 2, P_REL = 3, P_PREV1 = 4, P_PREV2 = 5, P_MPHI = 6, P_N = 8 };
-// status codes inside the kernel: 0 = still iterating, -1 = converged, else a gbmg_status
-enum { ST_ACTIVE = 0, ST_CONVERGED = -1 };
-
-struct BProb {
-  int L, nc;
-  Dims d[BMAXL];
-  float* r[BMAXL];
-  float* ea[BMAXL];
-  float* eb[BMAXL];
-  float* dv[BMAXL];
-  float* t[BMAXL];
-  const float* G;
-  float2* F;
-  float2* phi;   // double-float phi, and the second buffer of the fused update (phi2)
-  float2* phi2;
-  const double* src;
-  double* out;
-  int c0, nch;      // first level-0 chunk and count
-  unsigned fmask;   // bit l: level l runs the fused legs
-  int dffused;      // the finest level runs the fused double-float update (even nx)
-  int ls;           // first level of the single-CTA bottom cycle (levels ls .. L-1), 0: none
-};
-
-struct BDesc {
-  int count, maxL, degree, maxv;
-  int chunk[BMAXL];  // tile (chunk) size in cells per level
-  double tol;
-  float c1[16];
-  float ca[BMAXL][8];  // folded Chebyshev constants a = c2 D^-1 and b = a / h^2 per level and step
-  float cb[BMAXL][8];
-  float ih2[BMAXL];    // 1 / h_l^2
-  const legs::Coef* coef;       // folded Chebyshev constants per level (device)
-  const long long* doff[BMAXL];  // per level: prefix over problems of fused down-leg planes
-  const long long* uoff[BMAXL];  // per level: the same for the up leg
-  long long dtot[BMAXL], utot[BMAXL];
-  const int* dfoff;              // prefix over problems of fused double-float items
-  int dftot;
-  double* dfpart;                // per double-float item: partial sum of r^2
-  double* dfpart2;               // per double-float item: partial sum of (F - m)^2 (first residual)
-  unsigned perop;                // bit l: some problem runs level l per operation (not the coarsest)
-  unsigned coarse;               // bit l: some problem's coarsest level is l (outside a bottom cycle)
-  const SmallCycle* small;       // per problem: parameters of its bottom cycle (ls > 0)
-  int anysmall;                  // some problem runs a bottom cycle
-  int* phicur;                   // per problem: 0 = phi, 1 = phi2 holds the current iterate
-  BProb* p;
-  // chunk tables per level: problem index and first cell
-  int* cprob[BMAXL];
-  long long* cstart[BMAXL];
-  int nchunk[BMAXL];
-  double* part0;  // per level-0 chunk partials
-  double* part1;
-  double* sc;     // count * P_N scalars
-  int* status;    // count: ST_ACTIVE, then a gbmg_status
-  int* cycles;    // count
-  double* hist;   // count * 64
-  double* rel0;   // count
-  unsigned long long* tdone;  // count, %globaltimer at completion
-  unsigned long long* tstart;
-  int* any_active;
-};
-
-__device__ __forceinline__ unsigned long long globaltimer() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-  return t;
-}
 
 // (x, y, z) of cell i of one problem: 32-bit division (every problem holds fewer than
 // 2^31 cells, checked at mg_batch_create), two divisions per cell.
@@ -166,36 +91,6 @@ __device__ __forceinline__ void phase(const BDesc& B, int l, Want want, Op op) {
     const long long s1 = s0 + B.chunk[l] < n ? s0 + B.chunk[l] : n;
     for (long long i = s0 + threadIdx.x; i < s1; i += blockDim.x) op(P, l, i);
   }
-}
-
-// Level-0 phase with a per-chunk partial sum of the float returned by op.
-template <typename Op>
-__device__ __forceinline__ void phase0_sum(const BDesc& B, double* part, double* sh, bool all, Op op) {
-  for (int c = blockIdx.x; c < B.nchunk[0]; c += gridDim.x) {
-    const int pi = B.cprob[0][c];
-    if (!all && B.status[pi] != ST_ACTIVE) continue;
-    const BProb& P = B.p[pi];
-    const long long s0 = B.cstart[0][c];
-    const long long n = ncell(P.d[0]);
-    const long long s1 = s0 + B.chunk[0] < n ? s0 + B.chunk[0] : n;
-    DfAcc acc{0.f, 0.f};
-    for (long long i = s0 + threadIdx.x; i < s1; i += blockDim.x) op(P, i, acc);
-    const double b = block_sum_acc(acc, sh);
-    if (threadIdx.x == 0) part[c] = b;
-  }
-}
-
-__device__ __forceinline__ double chunk_total(const BDesc& B, const BProb& P, const double* part) {
-  double s = 0.0;
-  for (int k = 0; k < P.nch; ++k) s += part[P.c0 + k];
-  return s;
-}
-
-// level l of problem P runs the fused legs
-__device__ __forceinline__ bool lv_fused(const BProb& P, int l) { return (P.fmask >> l) & 1u; }
-// buffer holding the final correction of level l after its up leg
-__device__ __forceinline__ float* final_e(const BProb& P, int l) {
-  return (l < P.L - 1 && lv_fused(P, l)) ? P.eb[l] : P.ea[l];
 }
 
 // Fused phases: the (problem, tile, plane) list of level l, split evenly over the
@@ -607,8 +502,9 @@ struct gbmg_batch {
   unsigned long long* htime = nullptr;
   unsigned long long* htstart = nullptr;
   size_t res_bytes = 0;
-  // CUDA graph of one solve (copy-in, resets, the cooperative launch, copy-out),
-  // captured on a private stream and replayed while its key is unchanged
+  // CUDA graph of one solve (copy-in, resets, the phase kernels in a device-side loop or,
+  // where they do not apply, the cooperative launch, copy-out), captured on a private stream
+  // and replayed while its key is unchanged
   bool use_graph = false;
   cudaStream_t gstream = nullptr;
   cudaEvent_t gev[2] = {nullptr, nullptr};
@@ -621,6 +517,7 @@ struct gbmg_batch {
   const void* kern = nullptr;
   size_t smem = 0;
   char* mem2 = nullptr;
+  PhaseGraph phases;  // the graph form of a solve, where it applies
   ~gbmg_batch() {
     if (gexec) cudaGraphExecDestroy(gexec);
     if (mem2) cudaFree(mem2);
@@ -837,6 +734,7 @@ extern "C" gbmg_status mg_batch_create(gbmg_batch** out, gbmg_ctx* const* ctxs, 
   // shared memory (fused degrees only); those levels leave the fused and per-operation
   // phases
   std::vector<SmallCycle> small(count);
+  size_t bottom = 0;
   for (int i = 0; i < count; ++i) {
     const gbmg_ctx* c = b->ctx[i];
     BProb& P = b->hprob[i];
@@ -845,6 +743,7 @@ extern "C" gbmg_status mg_batch_create(gbmg_batch** out, gbmg_ctx* const* ctxs, 
         P.ls = l;
         D.anysmall = 1;
         b->smem = std::max(b->smem, small_cycle_smem(small[i]));
+        bottom = std::max(bottom, small_cycle_smem(small[i]));
         break;
       }
     const int top = P.ls > 0 ? P.ls : c->L - 1;  // levels below top are fused or per operation
@@ -938,6 +837,7 @@ extern "C" gbmg_status mg_batch_create(gbmg_batch** out, gbmg_ctx* const* ctxs, 
     }
   }
   gbmg_status st = build_tables(b);
+  if (st == GBMG_OK) st = b->phases.init(b->ctx, b->hprob, D, bottom);
   // persistent grid: every block resident at once (cooperative launch)
   if (st == GBMG_OK) st = max_blocks(b, b->blocks);
   if (st != GBMG_OK) {
@@ -999,15 +899,22 @@ extern "C" gbmg_status mg_batch_solve(gbmg_batch* b, const double* const* src_de
   D.tol = tol;
   D.maxv = max_vcycles < 0 ? 0 : max_vcycles;
   // the whole solve as one stream-ordered sequence
-  auto enqueue = [&](cudaStream_t st) -> gbmg_status {
+  auto copy_in = [&](cudaStream_t st) -> gbmg_status {
     TRY(cudaMemcpyAsync(D.p, b->hprob, sizeof(BProb) * b->count, cudaMemcpyHostToDevice, st));
     TRY(cudaMemsetAsync(D.status, 0, sizeof(int) * b->count, st));
     TRY(cudaMemsetAsync(D.cycles, 0, sizeof(int) * b->count, st));
-    void* args[] = {&D};
-    TRY(cudaLaunchCooperativeKernel(b->kern, dim3(b->blocks), dim3(BT), args, b->smem, st));
+    return GBMG_OK;
+  };
+  auto copy_out = [&](cudaStream_t st) -> gbmg_status {
     TRY(cudaMemcpyAsync(b->hstatus, D.status, b->res_bytes, cudaMemcpyDeviceToHost, st));
     TRY(cudaMemcpyAsync(b->hsc, D.sc, sizeof(double) * P_N * b->count, cudaMemcpyDeviceToHost, st));
     return GBMG_OK;
+  };
+  auto enqueue = [&](cudaStream_t st) -> gbmg_status {
+    TRYS(copy_in(st));
+    void* args[] = {&D};
+    TRY(cudaLaunchCooperativeKernel(b->kern, dim3(b->blocks), dim3(BT), args, b->smem, st));
+    return copy_out(st);
   };
   if (!b->use_graph) {
     TRYS(enqueue(b->stream));
@@ -1024,14 +931,23 @@ extern "C" gbmg_status mg_batch_solve(gbmg_batch* b, const double* const* src_de
         b->gexec = nullptr;
       }
       cudaGraph_t graph = nullptr;
-      TRY(cudaStreamBeginCapture(b->gstream, cudaStreamCaptureModeThreadLocal));
-      const gbmg_status cs = enqueue(b->gstream);
-      const cudaError_t ce = cudaStreamEndCapture(b->gstream, &graph);
-      if (cs != GBMG_OK) {
-        if (graph) cudaGraphDestroy(graph);
-        return cs;
+      if (b->phases.usable) {
+        const gbmg_status cs = b->phases.build(b->gstream, D, &graph, [&]() { return copy_in(b->gstream); },
+                                               [&]() { return copy_out(b->gstream); });
+        if (cs != GBMG_OK) {
+          if (graph) cudaGraphDestroy(graph);
+          return cs;
+        }
+      } else {
+        TRY(cudaStreamBeginCapture(b->gstream, cudaStreamCaptureModeThreadLocal));
+        const gbmg_status cs = enqueue(b->gstream);
+        const cudaError_t ce = cudaStreamEndCapture(b->gstream, &graph);
+        if (cs != GBMG_OK) {
+          if (graph) cudaGraphDestroy(graph);
+          return cs;
+        }
+        TRY(ce);
       }
-      TRY(ce);
       const cudaError_t ie = cudaGraphInstantiate(&b->gexec, graph, 0);
       cudaGraphDestroy(graph);
       TRY(ie);

@@ -28,8 +28,6 @@
 // tile's z stream starts at its own phase (tile_phase), so that neighbouring tiles
 // stream the same planes at about the same time and their shared halo rows are read
 // from DRAM about once.
-#include <type_traits>
-
 #include "legs.cuh"
 
 namespace gbmg {
@@ -79,45 +77,6 @@ k_up_fused(Dims d, const float* __restrict__ e_in, const float* __restrict__ ec,
 }
 
 // ------------------------------------------------------------------ launch
-
-// Tiles per degree: 64 x 32 cells; block sizes are multiples of 128 threads
-// (registers are granted to groups of four warps).  Down leg (degrees 1-3): columns of
-// R = 3 pairs, 512 threads: 16 warps per SM within 128 registers (0.554 ms at 512^3
-// against 0.595 with 4-pair columns in 384 threads, 12 warps at 168 registers: the leg
-// is bound by dependency latency, which more warps hide); degree 4 (halo 5) keeps 4-pair
-// columns, 384 threads and a 64 x 24 tile, which fit its shared memory.  Up leg: columns
-// of R = 4 pairs, 384 threads (even R makes each row's y parity, and with it the
-// prolongation's coarse-row pattern, a compile-time constant).
-template <int V>
-struct DownTile {
-  using T = typename std::conditional<(V >= 4), PTile<64, 24, V + 1, 384, 4>, PTile<64, 32, V + 1, 512, 3>>::type;
-};
-template <int V>
-struct UpTile {
-  using T = PTile<64, 32, V, 384, 4>;
-};
-
-template <int V>
-size_t down_smem() {
-  return (size_t)(V + 1) * 2 * DownTile<V>::T::PLANE * sizeof(float);
-}
-template <int V>
-size_t up_smem() {
-  using TL = typename UpTile<V>::T;
-  return ((size_t)V * 2 * TL::PLANE + 3 * PCoarse<TL>::CN) * sizeof(float);
-}
-
-Coef make_coef(const double* c1, const double* c2, int v, double h) {
-  Coef cf{};
-  for (int i = 0; i < v && i < 16; ++i) {
-    double a, b;
-    cheb_constants(c2[i], h, a, b);
-    cf.c1[i] = (float)c1[i];
-    cf.a[i] = (float)a;
-    cf.b[i] = (float)b;
-  }
-  return cf;
-}
 
 int sm_count() {
   static int n = 0;
