@@ -74,7 +74,7 @@ __device__ __forceinline__ V nsum_at(const V* u, Dims d, int x, int y, int z, lo
   const V yp = u[i + (long long)((y == d.ny - 1 ? 0 : y + 1) - y) * sy];
   const V zm = u[i + (long long)((z == 0 ? d.nz - 1 : z - 1) - z) * sz];
   const V zp = u[i + (long long)((z == d.nz - 1 ? 0 : z + 1) - z) * sz];
-  return nbr_sum(xm, xp, ym, yp, zm, zp);
+  return lap_sum(xm, xp, ym, yp, zm, zp, u[i]);
 }
 
 // Run `op(P, l, i)` over every cell of level l of every active problem for which
@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(BT, 1) k_batched_solve(BDesc B) {
             s = nsum_at(e, d, x, y, z, i);
           }
           float dd = from_zero ? 0.f : P.dv[lv][i];
-          eo[i] = cheb_step(c, P.r[lv][i], s, c, dd, a, b, c1);
+          eo[i] = cheb_step(c, P.r[lv][i], s, dd, a, b, c1);
           P.dv[lv][i] = dd;
         });
         cur_a = !cur_a;
@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(BT, 1) k_batched_solve(BDesc B) {
         const float* e = cur_a ? P.ea[lv] : P.eb[lv];
         int x, y, z;
         cell_xyz(d, i, x, y, z);
-        P.t[lv][i] = resid_from_sum(P.r[lv][i], nsum_at(e, d, x, y, z, i), e[i], ih2);
+        P.t[lv][i] = resid_from_sum(P.r[lv][i], nsum_at(e, d, x, y, z, i), ih2);
       });
       grid.sync();
       phase(B, l + 1, [&](const BProb& P, int lv) { return smoothed(P, lv - 1); },
@@ -361,7 +361,7 @@ __global__ void __launch_bounds__(BT, 1) k_batched_solve(BDesc B) {
                 float zv[3];
 #pragma unroll
                 for (int b = 0; b < 3; ++b)
-                  zv[b] = fw3(f[lin(df, xs[a], ys[b], zs[0])], f[lin(df, xs[a], ys[b], zs[1])],
+                  zv[b] = fw3z(f[lin(df, xs[a], ys[b], zs[0])], f[lin(df, xs[a], ys[b], zs[1])],
                               f[lin(df, xs[a], ys[b], zs[2])]);
                 yv[a] = fw3(zv[0], zv[1], zv[2]);
               }
@@ -432,7 +432,7 @@ __global__ void __launch_bounds__(BT, 1) k_batched_solve(BDesc B) {
           cell_xyz(d, i, x, y, z);
           const float c = e[i];
           float dd = k == 0 ? 0.f : P.dv[lv][i];
-          eo[i] = cheb_step(c, P.r[lv][i], nsum_at(e, d, x, y, z, i), c, dd, a, b, c1);
+          eo[i] = cheb_step(c, P.r[lv][i], nsum_at(e, d, x, y, z, i), dd, a, b, c1);
           P.dv[lv][i] = dd;
         });
         cur_a = !cur_a;
@@ -775,16 +775,8 @@ extern "C" gbmg_status mg_batch_create(gbmg_batch** out, gbmg_ctx* const* ctxs, 
     dfoff[i + 1] = dfoff[i] + items;
   }
   std::vector<legs::Coef> coef(maxL);
-  for (int l = 0; l < maxL; ++l) {
-    std::memset(&coef[l], 0, sizeof(legs::Coef));
-    for (int k = 0; k < D.degree && k < 16; ++k) {
-      double a, bb;
-      cheb_constants(ctxs[0]->cc2[k], (double)(1 << l), a, bb);
-      coef[l].c1[k] = (float)ctxs[0]->cc1[k];
-      coef[l].a[k] = (float)a;
-      coef[l].b[k] = (float)bb;
-    }
-  }
+  for (int l = 0; l < maxL; ++l)
+    coef[l] = legs::make_coef(ctxs[0]->cc1.data(), ctxs[0]->cc2.data(), D.degree, (double)(1 << l));
   {
     size_t off2 = 0;
     auto take2 = [&](size_t bytes) {

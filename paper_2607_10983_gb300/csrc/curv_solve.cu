@@ -263,7 +263,7 @@ extern "C" gbmg_status mg_set_geometry(gbmg_ctx* c, const double* psi_dev) {
     if (l == 0) {
       TRY(cudaMemcpyAsync(L.psi, psi_dev, (size_t)ncell(L.d) * sizeof(double), cudaMemcpyDeviceToDevice, c->stream));
     } else {
-      TRY(launch_restrict<double>(c->stream, c->lv[l - 1].d, c->lv[l - 1].psi, L.psi));
+      TRY(launch_restrict<double>(c->stream, c->lv[l - 1].d, c->lv[l - 1].psi, L.psi, true));
     }
     CurvCoefOut o;
     o.J = (float*)L.cc.J;
@@ -293,8 +293,8 @@ extern "C" gbmg_status mg_set_coefficients(gbmg_ctx* c, const float* J_dev, cons
     } else {
       // coarse coefficients: full-weighting restriction of the finer level's coefficients
       const Level& F = c->lv[l - 1];
-      TRY(launch_restrict<float>(c->stream, F.d, F.cc.J, (float*)L.cc.J));
-      for (int k = 0; k < 6; ++k) TRY(launch_restrict<float>(c->stream, F.d, F.cc.B[k], (float*)L.cc.B[k]));
+      TRY(launch_restrict<float>(c->stream, F.d, F.cc.J, (float*)L.cc.J, true));
+      for (int k = 0; k < 6; ++k) TRY(launch_restrict<float>(c->stream, F.d, F.cc.B[k], (float*)L.cc.B[k], true));
     }
   }
   TRYS(build_diag(c));

@@ -50,8 +50,8 @@ __device__ __forceinline__ Nbrs<V> load_nbrs(const V* __restrict__ u, Dims d, in
 }
 
 template <typename T>
-__device__ __forceinline__ T nsum(const Nbrs<T>& n) {
-  return nbr_sum(n.xm, n.xp, n.ym, n.yp, n.zm, n.zp);
+__device__ __forceinline__ T nsum(const Nbrs<T>& n, T c) {
+  return lap_sum(n.xm, n.xp, n.ym, n.yp, n.zm, n.zp, c);
 }
 
 template <typename T>
@@ -62,7 +62,7 @@ __global__ void k_apply(Dims d, const T* __restrict__ u, T* __restrict__ out, T 
   const int x = blockIdx.x * BX + threadIdx.x, y = blockIdx.y * BY + threadIdx.y, z = blockIdx.z;
   if (x >= d.nx || y >= d.ny) return;
   const long long i = lin(d, x, y, z);
-  out[i] = lap_from_sum(nsum(load_nbrs(u, d, x, y, z, i)), u[i], inv_h2);
+  out[i] = lap_from_sum(nsum(load_nbrs(u, d, x, y, z, i), u[i]), inv_h2);
 }
 
 template <typename T>
@@ -73,7 +73,7 @@ __global__ void k_residual(Dims d, const T* __restrict__ f, const T* __restrict_
   T r = T(0);
   if (x < d.nx && y < d.ny) {
     const long long i = lin(d, x, y, z);
-    r = resid_from_sum(f[i], nsum(load_nbrs(u, d, x, y, z, i)), u[i], inv_h2);
+    r = resid_from_sum(f[i], nsum(load_nbrs(u, d, x, y, z, i), u[i]), inv_h2);
     out[i] = r;
   }
   if (partials) {
@@ -92,7 +92,7 @@ __global__ void k_cheb_step(Dims d, const T* __restrict__ r, const T* __restrict
   const long long i = lin(d, x, y, z);
   const T c = e_in[i];
   T dv = c1 == T(0) ? T(0) : dvec[i];
-  e_out[i] = cheb_step(c, r[i], nsum(load_nbrs(e_in, d, x, y, z, i)), c, dv, a, b, c1);
+  e_out[i] = cheb_step(c, r[i], nsum(load_nbrs(e_in, d, x, y, z, i), c), dv, a, b, c1);
   dvec[i] = dv;
 }
 
@@ -103,12 +103,12 @@ __global__ void k_jacobi(Dims d, const T* __restrict__ r, const T* __restrict__ 
   if (x >= d.nx || y >= d.ny) return;
   const long long i = lin(d, x, y, z);
   const T c = e_in[i];
-  e_out[i] = jacobi_step(c, r[i], nsum(load_nbrs(e_in, d, x, y, z, i)), c, wa, wb);
+  e_out[i] = jacobi_step(c, r[i], nsum(load_nbrs(e_in, d, x, y, z, i), c), wa, wb);
 }
 
 // Full weighting, one thread per coarse cell: z-axis weights first, then y, then x
-// (the order the fused kernels use).
-template <typename T>
+// (the order the fused kernels use; ZS: the z weights as fw3z).
+template <typename T, bool ZS>
 __global__ void k_restrict(Dims df, const T* __restrict__ f, T* __restrict__ c) {
   const Dims dc{df.nx / 2, df.ny / 2, df.nz / 2};
   const int X = blockIdx.x * BX + threadIdx.x, Y = blockIdx.y * BY + threadIdx.y, Z = blockIdx.z;
@@ -125,8 +125,12 @@ __global__ void k_restrict(Dims df, const T* __restrict__ f, T* __restrict__ c) 
   for (int a = 0; a < 3; ++a) {
     T zv[3];
 #pragma unroll
-    for (int b = 0; b < 3; ++b)
-      zv[b] = fw3(f[lin(df, xs[a], ys[b], zs[0])], f[lin(df, xs[a], ys[b], zs[1])], f[lin(df, xs[a], ys[b], zs[2])]);
+    for (int b = 0; b < 3; ++b) {
+      const T z0 = f[lin(df, xs[a], ys[b], zs[0])], z1 = f[lin(df, xs[a], ys[b], zs[1])],
+              z2 = f[lin(df, xs[a], ys[b], zs[2])];
+      if constexpr (ZS) zv[b] = fw3z(z0, z1, z2);
+      else zv[b] = fw3(z0, z1, z2);
+    }
     yv[a] = fw3(zv[0], zv[1], zv[2]);
   }
   c[lin(dc, X, Y, Z)] = fw3(yv[0], yv[1], yv[2]);
@@ -434,9 +438,11 @@ cudaError_t launch_jacobi(cudaStream_t st, Dims d, const T* r, const T* e_in, T*
   return cudaGetLastError();
 }
 template <typename T>
-cudaError_t launch_restrict(cudaStream_t st, Dims fine, const T* f, T* c) {
+cudaError_t launch_restrict(cudaStream_t st, Dims fine, const T* f, T* c, bool geometry) {
   const Dims dc{fine.nx / 2, fine.ny / 2, fine.nz / 2};
-  k_restrict<T><<<cell_grid(dc), dim3(BX, BY), 0, st>>>(fine, f, c);
+  constexpr bool zs = sizeof(T) == 4;
+  if (zs && !geometry) k_restrict<T, zs><<<cell_grid(dc), dim3(BX, BY), 0, st>>>(fine, f, c);
+  else k_restrict<T, false><<<cell_grid(dc), dim3(BX, BY), 0, st>>>(fine, f, c);
   note_launch();
   return cudaGetLastError();
 }
@@ -535,7 +541,7 @@ cudaError_t launch_df_update(cudaStream_t st, long long n, float2* phi, const fl
   template cudaError_t launch_residual<T>(cudaStream_t, Dims, const T*, const T*, T*, T, double*);   \
   template cudaError_t launch_cheb_step<T>(cudaStream_t, Dims, const T*, const T*, T*, T*, T, T, T);  \
   template cudaError_t launch_jacobi<T>(cudaStream_t, Dims, const T*, const T*, T*, T, T);           \
-  template cudaError_t launch_restrict<T>(cudaStream_t, Dims, const T*, T*);                         \
+  template cudaError_t launch_restrict<T>(cudaStream_t, Dims, const T*, T*, bool);                         \
   template cudaError_t launch_prolong_add<T>(cudaStream_t, Dims, const T*, T*);                      \
   template cudaError_t launch_coarse_matvec<T>(cudaStream_t, int, const T*, const T*, T*);           \
   template cudaError_t launch_sum<T>(cudaStream_t, long long, const T*, double*, double*);           \

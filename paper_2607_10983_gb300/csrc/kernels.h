@@ -33,8 +33,9 @@ inline void cheb_constants(double c2, double h, double& a, double& b) {
   a = c2 * dinv;
   b = a * (1.0 / (h * h));
 }
+// geometry: a curvilinear level's coefficients (FP32 residuals add the z weights as fw3z)
 template <typename T>
-cudaError_t launch_restrict(cudaStream_t st, Dims fine, const T* f, T* c);
+cudaError_t launch_restrict(cudaStream_t st, Dims fine, const T* f, T* c, bool geometry = false);
 template <typename T>
 cudaError_t launch_prolong_add(cudaStream_t st, Dims coarse, const T* c, T* f);
 template <typename T>

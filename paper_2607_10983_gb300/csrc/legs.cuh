@@ -69,11 +69,9 @@ struct PPos {
   }
 };
 
-// Folded Chebyshev constants of one level: c1 and a = c2 D^-1, b = a / h^2 per step.
+// Folded Chebyshev constants of one level: c1, a = c2 D^-1 and -b = -a / h^2 per step.
 struct Coef {
-  float c1[16];
-  float a[16];
-  float b[16];
+  float c1[4], a[4], mb[4];
 };
 
 struct Sched {
@@ -109,6 +107,19 @@ __device__ __forceinline__ void st2(float* p, float2 v) { *reinterpret_cast<floa
 // advance by one plane per iteration (wrapped once at the end of the mesh), plus the
 // thread's fixed in-plane offsets; the coarse outputs a thread writes are fixed per
 // tile and computed once.  Meshes have fewer than 2^31 cells per plane.
+//
+// Instructions.  The legs are bound by issue and dependency latency, and a third of what they
+// executed were register moves and integer operations.  So the plane loop is unrolled by two
+// (buffers become constants; the value a window shift moves is the one the next plane
+// overwrites, so the shift is a renaming), and the state between planes is kept small enough
+// for that not to spill: a stage's window is its plane and z- - 6 c instead of two planes
+// (lap_sum, which also takes two operations off each stage's chain), the residual's z weights
+// one partial sum (fw3z), d_1 = e_1 is not stored, and the first step from zero is a r.  The
+// shifts of loaded values stand at the top of an iteration: at its end the wait for the load
+// came before the barrier (0.58 ms).  A few bytes of spill cost more than all of this gives
+// (up leg 0.95 ms at 40 bytes): the L1 beside the shared planes is small.
+// 512^3, degree 3: down 0.531 -> 0.445 ms, up 0.658 -> 0.539; 64^3: 14.5 -> 12.5 us each.
+// Prefetching planes to L2 two ahead: 0.471 ms down.
 
 template <int V, class TL>
 __device__ __forceinline__ void down_segment(Dims d, const float* __restrict__ r, float* __restrict__ e_out,
@@ -141,17 +152,16 @@ __device__ __forceinline__ void down_segment(Dims d, const float* __restrict__ r
   const float2 Z = bcast(0.f), MIH2 = bcast(-inv_h2);
 
   float2 rq[V + 1][R];              // rq[i][j] = r at plane t - i
-  float2 wp[V + 2][R], wc[V + 2][R];  // stage s input window: planes zp - 1, zp
-  float2 dh[V + 1][R];              // d_{s-1} at stage s's plane
-  float2 rsp[R], rsc[R];            // residual window
-  float2 rnext[R];
+  float2 wc[V + 2][R], wt[V + 2][R];  // stage s input at plane zp: e, and (e at zp - 1) - 6 e
+  float2 dh[V + 1][R];              // d_{s-1} at stage s's plane, s >= 3 (d_1 = e_1)
+  float2 rnext[R], zwp[R];          // z weights' partial sum (fw3z)
 #pragma unroll
   for (int j = 0; j < R; ++j) {
 #pragma unroll
     for (int i = 0; i <= V; ++i) rq[i][j] = Z, dh[i][j] = Z;
 #pragma unroll
-    for (int s = 0; s < V + 2; ++s) wp[s][j] = Z, wc[s][j] = Z;
-    rsp[j] = rsc[j] = Z;
+    for (int s = 0; s < V + 2; ++s) wt[s][j] = Z, wc[s][j] = Z;
+    zwp[j] = Z;
   }
   // the last coarse plane c = zend - 1 (a segment may end on an odd plane) is
   // written at t = c + V + 2
@@ -160,8 +170,9 @@ __device__ __forceinline__ void down_segment(Dims d, const float* __restrict__ r
   const float* rl = r + (size_t)zl * pst;
 #pragma unroll
   for (int j = 0; j < R; ++j) rnext[j] = ld2(rl + P.goff[j]);
-  for (int t = tb; t <= te; ++t) {
-    const int cur = (t - tb) & 1;
+  // one plane; CUR: its buffer (t - tb) & 1, a constant
+  auto step = [&](int t, auto CUR) {
+    const int cur = CUR;
     float* const bc = bs + (cur ? PLANE : 0);
     const float* const bp = bs + (cur ? 0 : PLANE);
 #pragma unroll
@@ -182,33 +193,27 @@ __device__ __forceinline__ void down_segment(Dims d, const float* __restrict__ r
     }
     float2 en[V + 1][R], dn[V + 1][R];
     // stage 1 (pointwise, e starts at zero): e_1 = d_1 = c2_0 D^-1 r
-    {
-      const float2 A = bcast(cf.a[0]), MB = bcast(-cf.b[0]), C1 = bcast(cf.c1[0]);
 #pragma unroll
-      for (int j = 0; j < R; ++j) {
-        float2 dd = Z;
-        en[1][j] = p_cheb(Z, rq[0][j], Z, Z, dd, A, MB, C1);
-        dn[1][j] = dd;
-        bc[j * WS] = en[1][j].x;
-        bc[j * WS + HALF] = en[1][j].y;
-      }
+    for (int j = 0; j < R; ++j) {
+      en[1][j] = p_mul(bcast(cf.a[0]), rq[0][j]);
+      bc[j * WS] = en[1][j].x;
+      bc[j * WS + HALF] = en[1][j].y;
     }
     // stages 2..V: Chebyshev steps with the stencil on e_{s-1}
 #pragma unroll
     for (int s = 2; s <= V; ++s) {
       const float* const sE = bp + (s - 2) * SP;
       float* const dE = bc + (s - 1) * SP;
-      const float2 A = bcast(cf.a[s - 1]), MB = bcast(-cf.b[s - 1]), C1 = bcast(cf.c1[s - 1]);
 #pragma unroll
       for (int j = 0; j < R; ++j) {
         const int o = j * WS;
         const float2 c = wc[s][j];
         const float2 ym = j > 0 ? wc[s][j - 1] : make_float2(sE[o - WS], sE[o - WS + HALF]);
         const float2 yp = j < R - 1 ? wc[s][j + 1] : make_float2(sE[o + WS], sE[o + WS + HALF]);
-        const float2 sn = p_nbr_sum(sE[o - 1 + HALF], sE[o + 1], c, ym, yp, wp[s][j], en[s - 1][j]);
-        float2 dd = dh[s][j];
-        en[s][j] = p_cheb(c, rq[s - 1][j], sn, c, dd, A, MB, C1);
-        dn[s][j] = dd;
+        const float2 sn = p_lap_sum(sE[o - 1 + HALF], sE[o + 1], c, ym, yp, wt[s][j], en[s - 1][j]);
+        const float2 q = p_fma(bcast(cf.mb[s - 1]), sn, p_mul(bcast(cf.a[s - 1]), rq[s - 1][j]));
+        dn[s][j] = p_fma(bcast(cf.c1[s - 1]), s == 2 ? c : dh[s][j], q);
+        en[s][j] = p_add(c, dn[s][j]);
         dE[o] = en[s][j].x;
         dE[o + HALF] = en[s][j].y;
       }
@@ -222,27 +227,33 @@ __device__ __forceinline__ void down_segment(Dims d, const float* __restrict__ r
           if (P.tmask >> j & 1u) st2(ez + P.goff[j], en[V][j]);
       }
     }
-    // residual stage at plane t - V, then z weights of the restriction at c = t - V - 1
+    // residual stage at plane c + 1 = t - V; on odd planes the z weights of the restriction
+    // at c
     {
       const float* const sE = bp + (V - 1) * SP;
       float* const zE = bc + V * SP;
       const int c = t - V - 1;
-      const bool cz = ((c & 1) == 0) && c >= z0 && c < zend;
+      float2 rn[R];
 #pragma unroll
       for (int j = 0; j < R; ++j) {
         const int o = j * WS;
         const float2 cc = wc[V + 1][j];
         const float2 ym = j > 0 ? wc[V + 1][j - 1] : make_float2(sE[o - WS], sE[o - WS + HALF]);
         const float2 yp = j < R - 1 ? wc[V + 1][j + 1] : make_float2(sE[o + WS], sE[o + WS + HALF]);
-        const float2 sn = p_nbr_sum(sE[o - 1 + HALF], sE[o + 1], cc, ym, yp, wp[V + 1][j], en[V][j]);
-        const float2 rn = p_resid(rq[V][j], sn, cc, MIH2);
-        if (cz) {
-          const float2 zw = p_fw3(rsp[j], rsc[j], rn);
-          zE[o] = zw.x;
-          zE[o + HALF] = zw.y;
+        const float2 sn = p_lap_sum(sE[o - 1 + HALF], sE[o + 1], cc, ym, yp, wt[V + 1][j], en[V][j]);
+        rn[j] = p_fma(MIH2, sn, rq[V][j]);
+      }
+      if ((c & 1) == 0) {
+#pragma unroll
+        for (int j = 0; j < R; ++j) {
+          const float2 zw = p_fma(bcast(0.25f), rn[j], zwp[j]);
+          zE[j * WS] = zw.x;
+          zE[j * WS + HALF] = zw.y;
+          zwp[j] = rn[j];
         }
-        rsp[j] = rsc[j];
-        rsc[j] = rn;
+      } else {
+#pragma unroll
+        for (int j = 0; j < R; ++j) zwp[j] = p_fma(bcast(0.25f), zwp[j], p_mul(bcast(0.5f), rn[j]));
       }
     }
     // coarse output from the z-weighted plane of the previous iteration: y weights
@@ -270,13 +281,19 @@ __device__ __forceinline__ void down_segment(Dims d, const float* __restrict__ r
     for (int j = 0; j < R; ++j) {
 #pragma unroll
       for (int s = 2; s <= V + 1; ++s) {
-        wp[s][j] = wc[s][j];
+        wt[s][j] = p_below(en[s - 1][j], wc[s][j]);
         wc[s][j] = en[s - 1][j];
       }
 #pragma unroll
-      for (int s = 2; s <= V; ++s) dh[s][j] = dn[s - 1][j];
+      for (int s = 3; s <= V; ++s) dh[s][j] = dn[s - 1][j];
     }
     __syncthreads();
+  };
+  for (int t = tb;; t += 2) {
+    step(t, std::integral_constant<int, 0>());
+    if (t == te) break;
+    step(t + 1, std::integral_constant<int, 1>());
+    if (t + 1 == te) break;
   }
 }
 
@@ -360,12 +377,11 @@ __device__ __forceinline__ void up_segment(Dims d, const float* __restrict__ e_i
   const int par0 = (H + P.pyb * R) & 1;
   const int cb0 = tid < TL::NCOL ? (floor_half(y0 - H + P.pyb * R) - CY0) * CW + P.px : 0;
   // coarse cells of the ring this thread loads: in-plane offset (-1: none) and ring offset
-  int cgo[CL], cso[CL];
+  int cgo[CL];
 #pragma unroll
   for (int i = 0; i < CL; ++i) {
     const int q = tid + i * NT;
     const int ci = q % CU, cj = q / CU;
-    cso[i] = cj * CW + ci;
     cgo[i] = q < CU * CH ? wrapmod(CX0 + ci, cnx) + wrapmod(CY0 + cj, cny) * cnx : -1;
   }
   // coarse planes: slot of plane Ku (Ku = floor(t / 2)) and the plane of the next load
@@ -374,15 +390,21 @@ __device__ __forceinline__ void up_segment(Dims d, const float* __restrict__ e_i
   int ks = mod3(K0);
   int kl = wrapmod(K0, cnz);
   const float* ecl = ec + (size_t)kl * cpst;
-  auto load_coarse = [&](float (&vals)[CL]) {
-#pragma unroll
-    for (int i = 0; i < CL; ++i) vals[i] = cgo[i] >= 0 ? __ldg(ecl + cgo[i]) : 0.f;
-  };
-  auto store_coarse = [&](int slot, const float (&vals)[CL]) {
+  // asynchronous copies of plane kl's cells into a ring slot: through registers they and the
+  // kept ring offsets cost the six registers by which the unrolled loop spilled
+  auto copy_coarse = [&](int slot) {
+    int tq = tid;
+    asm volatile("" : "+r"(tq));
     float* const dst = cring + slot * CN;
 #pragma unroll
-    for (int i = 0; i < CL; ++i)
-      if (cgo[i] >= 0) dst[cso[i]] = vals[i];
+    for (int i = 0; i < CL; ++i) {
+      const int q = tq + i * NT, cj = q / CU;
+      if (cgo[i] >= 0) {
+        const unsigned sa = (unsigned)__cvta_generic_to_shared(dst + cj * CW + (q - cj * CU));
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(sa), "l"(ecl + cgo[i]) : "memory");
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
   };
   auto next_coarse = [&]() {
     if (++kl == cnz) {
@@ -395,54 +417,53 @@ __device__ __forceinline__ void up_segment(Dims d, const float* __restrict__ e_i
   const float2 Z = bcast(0.f);
 
   float2 rq[V + 1][R];
-  float2 wp[V + 1][R], wc[V + 1][R];
+  float2 wc[V + 1][R], wt[V + 1][R];  // stage s input at plane t - s: e, and (e below) - 6 e
   float2 dh[V + 1][R];
   float2 rnext[R], enext[R];
 #pragma unroll
   for (int j = 0; j < R; ++j) {
 #pragma unroll
-    for (int i = 0; i <= V; ++i) rq[i][j] = Z, dh[i][j] = Z, wp[i][j] = Z, wc[i][j] = Z;
+    for (int i = 0; i <= V; ++i) rq[i][j] = Z, dh[i][j] = Z, wt[i][j] = Z, wc[i][j] = Z;
   }
   int zl = wrapmod(tb, d.nz);                   // plane of the latest fine loads
   size_t ol = (size_t)zl * pst;
   {
-    float cv[CL];
-    load_coarse(cv);
-    store_coarse(ks, cv);
+    copy_coarse(ks);
     next_coarse();
-    load_coarse(cv);
-    store_coarse(ks == 2 ? 0 : ks + 1, cv);
+    copy_coarse(ks == 2 ? 0 : ks + 1);
     next_coarse();
+    asm volatile("cp.async.wait_all;" ::: "memory");
   }
 #pragma unroll
   for (int j = 0; j < R; ++j) {
-    rnext[j] = ld2(r + ol + P.goff[j]);
+    rnext[j] = Z;
     enext[j] = ld2(e_in + ol + P.goff[j]);
   }
   __syncthreads();
-  for (int t = tb; t <= te; ++t) {
-    const int cur = (t - tb) & 1;
+  // one plane; CUR: its buffer (t - tb) & 1, a constant
+  auto step = [&](int t, auto CUR) {
+    const int cur = CUR;
     float* const bc = bs + (cur ? PLANE : 0);
     const float* const bp = bs + (cur ? 0 : PLANE);
     const bool zodd = (t & 1) != 0;
     if (!zodd && t != tb) ks = ks == 2 ? 0 : ks + 1;   // Ku advanced
     const int ks1 = ks == 2 ? 0 : ks + 1;
     float2 en[V + 1][R], dn[V + 1][R];
-    // next coarse plane (needed from the next even t on), stored at the end of this iteration
-    float cv[CL];
-    const bool need_c = zodd && t < te;
-    if (need_c) {
-      load_coarse(cv);
+    // next coarse plane, needed in the iteration after the next
+    if (zodd && t < te) {
+      copy_coarse(ks1 == 2 ? 0 : ks1 + 1);
       next_coarse();
     }
 #pragma unroll
     for (int j = 0; j < R; ++j) {
 #pragma unroll
-      for (int i = V; i > 0; --i) rq[i][j] = rq[i - 1][j];
-      rq[0][j] = rnext[j];
+      for (int i = V; i > 1; --i) rq[i][j] = rq[i - 1][j];
+      rq[1][j] = rnext[j];
       en[0][j] = enext[j];
     }
     if (t < te) {
+#pragma unroll
+      for (int j = 0; j < R; ++j) rnext[j] = ld2(r + ol + P.goff[j]);
       if (++zl == d.nz) {
         zl = 0;
         ol = 0;
@@ -450,10 +471,7 @@ __device__ __forceinline__ void up_segment(Dims d, const float* __restrict__ e_i
         ol += pst;
       }
 #pragma unroll
-      for (int j = 0; j < R; ++j) {
-        rnext[j] = ld2(r + ol + P.goff[j]);
-        enext[j] = ld2(e_in + ol + P.goff[j]);
-      }
+      for (int j = 0; j < R; ++j) enext[j] = ld2(e_in + ol + P.goff[j]);
     }
     // stage 0: e_0 = e + P e_c (pointwise)
     {
@@ -476,17 +494,16 @@ __device__ __forceinline__ void up_segment(Dims d, const float* __restrict__ e_i
     for (int s = 1; s <= V; ++s) {
       const float* const sE = bp + (s - 1) * SP;
       float* const dE = bc + s * SP;
-      const float2 A = bcast(cf.a[s - 1]), MB = bcast(-cf.b[s - 1]), C1 = bcast(cf.c1[s - 1]);
 #pragma unroll
       for (int j = 0; j < R; ++j) {
         const int o = j * WS;
         const float2 c = wc[s][j];
         const float2 ym = j > 0 ? wc[s][j - 1] : make_float2(sE[o - WS], sE[o - WS + HALF]);
         const float2 yp = j < R - 1 ? wc[s][j + 1] : make_float2(sE[o + WS], sE[o + WS + HALF]);
-        const float2 sn = p_nbr_sum(sE[o - 1 + HALF], sE[o + 1], c, ym, yp, wp[s][j], en[s - 1][j]);
-        float2 dd = s == 1 ? Z : dh[s][j];
-        en[s][j] = p_cheb(c, rq[s][j], sn, c, dd, A, MB, C1);
-        dn[s][j] = dd;
+        const float2 sn = p_lap_sum(sE[o - 1 + HALF], sE[o + 1], c, ym, yp, wt[s][j], en[s - 1][j]);
+        const float2 q = p_fma(bcast(cf.mb[s - 1]), sn, p_mul(bcast(cf.a[s - 1]), rq[s][j]));
+        dn[s][j] = s == 1 ? q : p_fma(bcast(cf.c1[s - 1]), dh[s][j], q);
+        en[s][j] = p_add(c, dn[s][j]);
         if (s < V) {
           dE[o] = en[s][j].x;
           dE[o + HALF] = en[s][j].y;
@@ -506,14 +523,20 @@ __device__ __forceinline__ void up_segment(Dims d, const float* __restrict__ e_i
     for (int j = 0; j < R; ++j) {
 #pragma unroll
       for (int s = 1; s <= V; ++s) {
-        wp[s][j] = wc[s][j];
+        wt[s][j] = p_below(en[s - 1][j], wc[s][j]);
         wc[s][j] = en[s - 1][j];
       }
 #pragma unroll
       for (int s = 2; s <= V; ++s) dh[s][j] = dn[s - 1][j];
     }
-    if (need_c) store_coarse(ks1 == 2 ? 0 : ks1 + 1, cv);
+    if (!zodd) asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
+  };
+  for (int t = tb;; t += 2) {
+    step(t, std::integral_constant<int, 0>());
+    if (t == te) break;
+    step(t + 1, std::integral_constant<int, 1>());
+    if (t + 1 == te) break;
   }
 }
 
@@ -521,12 +544,12 @@ __device__ __forceinline__ void up_segment(Dims d, const float* __restrict__ e_i
 
 // Tiles per degree: 64 x 32 cells; block sizes are multiples of 128 threads
 // (registers are granted to groups of four warps).  Down leg (degrees 1-3): columns of
-// R = 3 pairs, 512 threads: 16 warps per SM within 128 registers (0.554 ms at 512^3
-// against 0.595 with 4-pair columns in 384 threads, 12 warps at 168 registers: the leg
-// is bound by dependency latency, which more warps hide); degree 4 (halo 5) keeps 4-pair
-// columns, 384 threads and a 64 x 24 tile, which fit its shared memory.  Up leg: columns
-// of R = 4 pairs, 384 threads (even R makes each row's y parity, and with it the
-// prolongation's coarse-row pattern, a compile-time constant).
+// R = 3 pairs, 512 threads, 16 warps per SM within 128 registers (0.450 ms at 512^3
+// against 0.468 with 4-pair columns in 384 threads and 0.484 with 6-pair columns in 256);
+// degree 4 (halo 5) keeps 4-pair columns, 384 threads and a 64 x 24 tile, which fit its
+// shared memory.  Up leg: columns of R = 4 pairs, 384 threads (even R makes each row's y
+// parity, and with it the prolongation's coarse-row pattern, a compile-time constant;
+// 6-pair columns in 256 threads 0.552 against 0.539 ms).
 template <int V>
 struct DownTile {
   using T = typename std::conditional<(V >= 4), PTile<64, 24, V + 1, 384, 4>, PTile<64, 32, V + 1, 512, 3>>::type;
@@ -548,12 +571,12 @@ size_t up_smem() {
 
 inline Coef make_coef(const double* c1, const double* c2, int v, double h) {
   Coef cf{};
-  for (int i = 0; i < v && i < 16; ++i) {
+  for (int i = 0; i < v && i < 4; ++i) {
     double a, b;
     cheb_constants(c2[i], h, a, b);
     cf.c1[i] = (float)c1[i];
     cf.a[i] = (float)a;
-    cf.b[i] = (float)b;
+    cf.mb[i] = -(float)b;
   }
   return cf;
 }

@@ -32,27 +32,12 @@ __device__ __forceinline__ float2 p_fma(float2 a, float2 b, float2 c) {
 }
 __device__ __forceinline__ float2 bcast(float v) { return make_float2(v, v); }
 
-// nbr_sum of the pair: the x neighbours of the even cell are (xm, c.y), those of
-// the odd cell (c.x, xp); then y, then z, in the order of the scalar nbr_sum.
-__device__ __forceinline__ float2 p_nbr_sum(float xm, float xp, float2 c, float2 ym, float2 yp, float2 zm,
-                                            float2 zp) {
-  float2 s = make_float2(t_add(xm, c.y), t_add(c.x, xp));
-  s = p_add(s, p_add(ym, yp));
-  return p_add(s, p_add(zm, zp));
-}
-// cheb_step on a pair (folded constants a, -b, c1 broadcast)
-__device__ __forceinline__ float2 p_cheb(float2 e, float2 r, float2 s, float2 c, float2& d, float2 a, float2 mb,
-                                         float2 c1) {
-  const float2 q = p_fma(mb, p_fma(bcast(-6.f), c, s), p_mul(a, r));
-  d = p_fma(c1, d, q);
-  return p_add(e, d);
-}
-// resid_from_sum on a pair (mih2 = -1/h^2 broadcast)
-__device__ __forceinline__ float2 p_resid(float2 r, float2 s, float2 c, float2 mih2) {
-  return p_fma(mih2, p_fma(bcast(-6.f), c, s), r);
-}
-__device__ __forceinline__ float2 p_fw3(float2 a, float2 b, float2 c) {
-  return p_fma(bcast(0.25f), p_add(a, c), p_mul(bcast(0.5f), b));
+// lap_sum of the pair: the x neighbours of the even cell are (xm, c.y), those of the odd
+// cell (c.x, xp); t = z- - 6 c (p_below).
+__device__ __forceinline__ float2 p_below(float2 c, float2 zm) { return p_fma(bcast(-6.f), c, zm); }
+__device__ __forceinline__ float2 p_lap_sum(float xm, float xp, float2 c, float2 ym, float2 yp, float2 t, float2 zp) {
+  const float2 s = make_float2(t_add(xm, c.y), t_add(c.x, xp));
+  return p_add(p_add(p_add(s, p_add(ym, yp)), t), zp);
 }
 __device__ __forceinline__ float2 p_half_sum(float2 a, float2 b) { return p_mul(bcast(0.5f), p_add(a, b)); }
 
@@ -96,7 +81,7 @@ struct PAcc {
   }
 };
 // df_resid of stencil.cuh on a pair: r = (F - m) - (sum of neighbours - 6 c), the hi
-// parts summed error-free, the lo parts in plain FP32; x neighbours as in p_nbr_sum.
+// parts summed error-free, the lo parts in plain FP32; x neighbours as in p_lap_sum.
 __device__ __forceinline__ float2 p_df_resid(DF2 c, float xm_hi, float xm_lo, float xp_hi, float xp_lo, DF2 ym,
                                              DF2 yp, DF2 zm, DF2 zp, DF2 f, DF2 m) {
   const float2 xmh = make_float2(xm_hi, c.hi.x), xph = make_float2(c.hi.y, xp_hi);

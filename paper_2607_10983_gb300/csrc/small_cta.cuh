@@ -67,7 +67,7 @@ __device__ __forceinline__ void load_item(const Item& I, const float* u, float (
   }
 #pragma unroll
   for (int q = 0; q < 4; ++q)
-    s[q] = nbr_sum(xm[q], xp[q], ym[q], yp[q], q ? c[q - 1] : lo, q + 1 < I.cnt && q < 3 ? c[q + 1] : hi);
+    s[q] = lap_sum(xm[q], xp[q], ym[q], yp[q], q ? c[q - 1] : lo, q + 1 < I.cnt && q < 3 ? c[q + 1] : hi, c[q]);
 }
 
 // e_out = V-cycle(r_in) on level 0 of P; sm: small_cycle_smem(P) bytes.
@@ -107,7 +107,7 @@ __device__ __forceinline__ void vcycle(const SmallCycle& P, const float* __restr
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           float t = 0.f;
-          const float e = cheb_step(0.f, r[q], 0.f, 0.f, t, a, b, c1);
+          const float e = cheb_step(0.f, r[q], 0.f, t, a, b, c1);
           dv[q] = t;
           if (q >= I.cnt) continue;
           if (load) R[I.i[q]] = r[q];
@@ -143,7 +143,7 @@ __device__ __forceinline__ void vcycle(const SmallCycle& P, const float* __restr
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           if (c1 == 0.f) dv[q] = 0.f;
-          e[q] = cheb_step(c[q], r[q], s[q], c[q], dv[q], a, b, c1);
+          e[q] = cheb_step(c[q], r[q], s[q], dv[q], a, b, c1);
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -173,7 +173,7 @@ __device__ __forceinline__ void vcycle(const SmallCycle& P, const float* __restr
         load_item(I, E, c, s);
 #pragma unroll
         for (int q = 0; q < 4; ++q)
-          if (q < I.cnt) E2[I.i[q]] = resid_from_sum(r[q], s[q], c[q], ih2);
+          if (q < I.cnt) E2[I.i[q]] = resid_from_sum(r[q], s[q], ih2);
       }
       __syncthreads();
       const float* const T = E2;
@@ -202,8 +202,8 @@ __device__ __forceinline__ void vcycle(const SmallCycle& P, const float* __restr
         float yv[3];
 #pragma unroll
         for (int a = 0; a < 3; ++a)
-          yv[a] = fw3(fw3(v[a][0][0], v[a][0][1], v[a][0][2]), fw3(v[a][1][0], v[a][1][1], v[a][1][2]),
-                      fw3(v[a][2][0], v[a][2][1], v[a][2][2]));
+          yv[a] = fw3(fw3z(v[a][0][0], v[a][0][1], v[a][0][2]), fw3z(v[a][1][0], v[a][1][1], v[a][1][2]),
+                      fw3z(v[a][2][0], v[a][2][1], v[a][2][2]));
         Rc[i] = fw3(yv[0], yv[1], yv[2]);
       }
       I.set(dc, tid);

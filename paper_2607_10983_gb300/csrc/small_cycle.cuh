@@ -27,7 +27,7 @@ __device__ __forceinline__ Nbrs6<float> nbrs(const float* u, Dims d, int x, int 
   n.zp = u[i + ((z == d.nz - 1 ? 0 : z + 1) - z) * sz];
   return n;
 }
-__device__ __forceinline__ float nsum6(const Nbrs6<float>& n) { return nbr_sum(n.xm, n.xp, n.ym, n.yp, n.zm, n.zp); }
+__device__ __forceinline__ float nsum6(const Nbrs6<float>& n, float c) { return lap_sum(n.xm, n.xp, n.ym, n.yp, n.zm, n.zp, c); }
 
 
 // Cells i = tid, tid + nt, ... of a level with their (x, y, z), advanced by mixed-radix
@@ -108,7 +108,7 @@ __device__ __forceinline__ void block_vcycle_n(const SmallCycle& P, const float*
         const int i = w.i;
         const float c = E[i];
         float dv = c1 == 0.f ? 0.f : DV[i];
-        E2[i] = cheb_step(c, R[i], nsum6(nbrs(E, d, w.x, w.y, w.z, i)), c, dv, a, b, c1);
+        E2[i] = cheb_step(c, R[i], nsum6(nbrs(E, d, w.x, w.y, w.z, i), c), dv, a, b, c1);
         DV[i] = dv;
       }
       __syncthreads();
@@ -129,7 +129,7 @@ __device__ __forceinline__ void block_vcycle_n(const SmallCycle& P, const float*
       float* T = sm + oT[l];
       const float ih2 = P.inv_h2[l];
       for (Walk w(d, tid, nt); w.i < n; w.next(d, nt))
-        T[w.i] = resid_from_sum(R[w.i], nsum6(nbrs(E, d, w.x, w.y, w.z, w.i)), E[w.i], ih2);
+        T[w.i] = resid_from_sum(R[w.i], nsum6(nbrs(E, d, w.x, w.y, w.z, w.i), E[w.i]), ih2);
     }
     __syncthreads();
     const Dims dc = P.d[l + 1];
@@ -152,7 +152,7 @@ __device__ __forceinline__ void block_vcycle_n(const SmallCycle& P, const float*
           float zv[3];
 #pragma unroll
           for (int b = 0; b < 3; ++b)
-            zv[b] = fw3(T[(int)lin(d, xs[a], ys[b], zs[0])], T[(int)lin(d, xs[a], ys[b], zs[1])],
+            zv[b] = fw3z(T[(int)lin(d, xs[a], ys[b], zs[0])], T[(int)lin(d, xs[a], ys[b], zs[1])],
                         T[(int)lin(d, xs[a], ys[b], zs[2])]);
           yv[a] = fw3(zv[0], zv[1], zv[2]);
         }

@@ -16,50 +16,56 @@ __device__ __forceinline__ double t_mul(double a, double b) { return __dmul_rn(a
 __device__ __forceinline__ float t_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double t_fma(double a, double b, double c) { return __fma_rn(a, b, c); }
 
-// Sum of the six face neighbours, in the fixed order (x-, x+), (y-, y+), (z-, z+).
+// Sum of the six face neighbours minus six times the cell, ((x- + x+) + (y- + y+)) +
+// (z- - 6 c) + z+: a kernel that streams planes upwards forms z- - 6 c one plane ahead (one
+// value to keep instead of z-) and adds z+, the value it has just computed, last, so that a
+// smoothing step is four dependent operations long (six with (z- + z+) formed first).
 template <typename T>
-__device__ __forceinline__ T nbr_sum(T xm, T xp, T ym, T yp, T zm, T zp) {
-  T s = t_add(xm, xp);
-  s = t_add(s, t_add(ym, yp));
-  s = t_add(s, t_add(zm, zp));
-  return s;
+__device__ __forceinline__ T lap_sum(T xm, T xp, T ym, T yp, T zm, T zp, T c) {
+  return t_add(t_add(t_add(t_add(xm, xp), t_add(ym, yp)), t_fma(T(-6), c, zm)), zp);
 }
 
-// (A_l u)_i = (sum of neighbours - 6 u_i) / h_l^2   (Sec. 2.1, Eq. linsys)
+// (A_l u)_i = (sum of neighbours - 6 u_i) / h_l^2   (Sec. 2.1, Eq. linsys); s = lap_sum
 template <typename T>
-__device__ __forceinline__ T lap_from_sum(T s, T c, T inv_h2) {
-  return t_mul(t_fma(T(-6), c, s), inv_h2);
+__device__ __forceinline__ T lap_from_sum(T s, T inv_h2) {
+  return t_mul(s, inv_h2);
 }
 
-// r - A_l u = r - (s - 6c) / h^2
+// r - A_l u = r - s / h^2
 template <typename T>
-__device__ __forceinline__ T resid_from_sum(T r, T s, T c, T inv_h2) {
-  return t_fma(-inv_h2, t_fma(T(-6), c, s), r);
+__device__ __forceinline__ T resid_from_sum(T r, T s, T inv_h2) {
+  return t_fma(-inv_h2, s, r);
 }
 
 // One Chebyshev step (Sec. 2.3, Eq. flat_chebyshev, semi-iteration form)
 //   z = D^-1 (r - A e);  d = c1 d + c2 z;  e += d,
 // evaluated with the constants folded: a = c2 D^-1, b = a / h^2 (each rounded once
-// on the host), q = a r - b (s - 6c), d = c1 d + q.  The first step of a pass has
+// on the host), q = a r - b s, d = c1 d + q.  The first step of a pass has
 // c1 = 0 (d = z / theta).  Returns the new e, updates d.
 template <typename T>
-__device__ __forceinline__ T cheb_step(T e, T r, T s, T c, T& d, T a, T b, T c1) {
-  const T q = t_fma(-b, t_fma(T(-6), c, s), t_mul(a, r));
+__device__ __forceinline__ T cheb_step(T e, T r, T s, T& d, T a, T b, T c1) {
+  const T q = t_fma(-b, s, t_mul(a, r));
   d = t_fma(c1, d, q);
   return t_add(e, d);
 }
 
 // Weighted Jacobi (Sec. 2.3, Eq. flat_jacobi): e + omega D^-1 (r - A e), with
-// wa = omega D^-1 and wb = wa / h^2: e + wa r - wb (s - 6c).
+// wa = omega D^-1 and wb = wa / h^2: e + wa r - wb s.
 template <typename T>
-__device__ __forceinline__ T jacobi_step(T e, T r, T s, T c, T wa, T wb) {
-  return t_fma(-wb, t_fma(T(-6), c, s), t_fma(wa, r, e));
+__device__ __forceinline__ T jacobi_step(T e, T r, T s, T wa, T wb) {
+  return t_fma(-wb, s, t_fma(wa, r, e));
 }
 
 // One axis of full weighting: (a + c)/4 + b/2 (Appendix B).
 template <typename T>
 __device__ __forceinline__ T fw3(T a, T b, T c) {
   return t_fma(T(0.25), t_add(a, c), t_mul(T(0.5), b));
+}
+
+// The z axis of full weighting in FP32 restrictions of the flat operator's residual: the terms
+// in the order of the planes, so that a kernel that streams planes keeps one partial sum.
+__device__ __forceinline__ float fw3z(float a, float b, float c) {
+  return t_fma(0.25f, c, t_fma(0.25f, a, t_mul(0.5f, b)));
 }
 
 // One axis of trilinear interpolation between neighbouring coarse nodes.
