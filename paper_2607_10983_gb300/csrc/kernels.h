@@ -106,6 +106,11 @@ cudaError_t launch_down_fused(cudaStream_t st, int degree, Dims d, const float* 
 // e_out = Chebyshev post-smoothing of A e = r starting from e_in + P ec.
 cudaError_t launch_up_fused(cudaStream_t st, int degree, Dims d, const float* e_in, const float* ec,
                             const float* r, float* e_out, double h, const double* c1, const double* c2);
+// The same legs for small levels, degrees 1 to 3 (block_legs.cu).
+cudaError_t launch_block_down(cudaStream_t st, int degree, Dims d, const float* r, float* e, float* rc, double h,
+                              const double* c1, const double* c2);
+cudaError_t launch_block_up(cudaStream_t st, int degree, Dims d, const float* e_in, const float* ec, const float* r,
+                            float* e_out, double h, const double* c1, const double* c2);
 // Finest level: phi_out = phi_in + e (double-float), r_out = F - m - A phi_out, with block partials
 // of ||r_out||^2, sum(phi_out) and (pf2 nullable) ||F - m||^2, df_update_residual_partials(d) each.
 // e NULL: no update (phi_out may then be NULL: not written).

@@ -88,13 +88,20 @@ int sm_count() {
   return n;
 }
 
+// A CTA whose range crosses a tile's end runs two segments, each with its warm-up planes.
+// Where that costs more than leaving some SMs idle, every tile gets the same number of CTAs
+// (six tiles of 80^3 or 96^3 on 150 CTAs: 21 -> 13 us; 512^3 keeps all SMs).
 template <class TL>
-Sched make_sched(Dims d, int& ctas) {
+Sched make_sched(Dims d, int warm, int& ctas) {
   Sched sc;
   sc.tiles_x = (d.nx + TL::TX - 1) / TL::TX;
-  sc.total = (long long)sc.tiles_x * ((d.ny + TL::TY - 1) / TL::TY) * d.nz;
-  const long long g = sc.total < sm_count() ? sc.total : sm_count();
+  const long long tiles = (long long)sc.tiles_x * ((d.ny + TL::TY - 1) / TL::TY);
+  sc.total = tiles * d.nz;
+  const long long sms = sm_count();
+  const long long g = sc.total < sms ? sc.total : sms;
+  const long long k = sms / tiles < d.nz ? sms / tiles : d.nz;  // CTAs per tile
   ctas = (int)g;
+  if (k > 0 && g % tiles != 0 && (d.nz + k - 1) / k + warm < (sc.total + g - 1) / g + 2 * warm) ctas = (int)(k * tiles);
   return sc;
 }
 
@@ -109,7 +116,7 @@ cudaError_t down_v(cudaStream_t st, Dims d, const float* r, float* e, float* rc,
     attr = true;
   }
   int ctas = 0;
-  const Sched sc = make_sched<TL>(d, ctas);
+  const Sched sc = make_sched<TL>(d, 2 * V + 3, ctas);
   k_down_fused<V, TL><<<ctas, TL::NT, sm, st>>>(d, r, e, rc, sc, ih2, cf);
   note_launch();
   return cudaGetLastError();
@@ -127,7 +134,7 @@ cudaError_t up_v(cudaStream_t st, Dims d, const float* e_in, const float* ec, co
     attr = true;
   }
   int ctas = 0;
-  const Sched sc = make_sched<TL>(d, ctas);
+  const Sched sc = make_sched<TL>(d, 2 * V, ctas);
   k_up_fused<V, TL><<<ctas, TL::NT, sm, st>>>(d, e_in, ec, r, e_out, sc, ih2, cf);
   note_launch();
   return cudaGetLastError();

@@ -124,23 +124,27 @@ gbmg_status vcycle_unfused(gbmg_ctx* c, int l, T*& e, T*& eo, const T* r) {
   return GBMG_OK;
 }
 
-// Levels of at least 2^18 cells (64^3) use the temporally blocked kernels; below
-// that a level visit is latency-bound and the one-kernel-per-operation chain is as
-// fast.  Measured on the 512^3 / 256^3 warm sequences: thresholds 2^23 / 2^21 / 2^18
-// gave 64.0 / 65.3 / 65.3 and 280 / 303 / 309 solves/s.
+// Levels of at least 2^18 cells (64^3) use the z-streaming legs (the two legs at degree 3:
+// 64^3 19.7 us, in blocks 21.2; 80^3 26.6 and 35; 48^3 20.2 and 12.1).
 constexpr long long kFusedMinCells = 1ll << 18;
 bool level_fused(const gbmg_ctx* c, int l) {
   const Dims d = c->lv[l].d;
   return c->o.fused && l < c->L - 1 && d.nx >= 16 && d.ny >= 16 && d.nz >= 16 &&
          (ncell(d) >= kFusedMinCells || c->fused_all);
 }
+// Smaller levels above the bottom cycle run each leg in blocks held in shared memory (32^3,
+// degree 3: 8.3 us against about 18 for the chain of seven kernels and a memset).
+bool level_blocked(const gbmg_ctx* c, int l) {
+  return c->o.fused && l < c->L - 1 && c->o.degree <= 3 && !level_fused(c, l) && !small_cycle_from(c, l, nullptr);
+}
 
-// V-cycle in FP32 with the temporally blocked kernels on large levels (one launch per
-// level visit on each leg) and the one-kernel-per-operation path below them.  e
+// V-cycle in FP32, one launch per level visit and leg down to the bottom cycle (degree 4 and
+// coarsest levels: the one-kernel-per-operation path below the large levels).  e
 // receives the pointer to the level's correction.
 gbmg_status vcycle_fused(gbmg_ctx* c, int l, float*& e, const float* r) {
   const Level& L = c->lv[l];
-  if (!level_fused(c, l)) {
+  const bool blocked = level_blocked(c, l);
+  if (!blocked && !level_fused(c, l)) {
     float* ee = (float*)L.e;
     float* eo = (float*)L.e2;
     if (l < c->L - 1 && !small_cycle_from(c, l, nullptr))
@@ -152,16 +156,16 @@ gbmg_status vcycle_fused(gbmg_ctx* c, int l, float*& e, const float* r) {
   const Level& C = c->lv[l + 1];
   {
     ProfScope ps(c, l == 0 ? GBMG_PROF_DOWN0 : GBMG_PROF_OFF);
-    TRY(launch_down_fused(c->stream, c->o.degree, L.d, r, (float*)L.e, (float*)C.r, L.h, c->cc1.data(),
-                          c->cc2.data()));
+    TRY((blocked ? launch_block_down : launch_down_fused)(c->stream, c->o.degree, L.d, r, (float*)L.e, (float*)C.r,
+                                                          L.h, c->cc1.data(), c->cc2.data()));
   }
   float* ce = nullptr;
   TRYS(vcycle_fused(c, l + 1, ce, (const float*)C.r));
   TRYS(store_coarse_correction(c, l + 1, ce));
   {
     ProfScope ps(c, l == 0 ? GBMG_PROF_UP0 : GBMG_PROF_OFF);
-    TRY(launch_up_fused(c->stream, c->o.degree, L.d, (const float*)L.e, ce, r, (float*)L.e2, L.h,
-                        c->cc1.data(), c->cc2.data()));
+    TRY((blocked ? launch_block_up : launch_up_fused)(c->stream, c->o.degree, L.d, (const float*)L.e, ce, r,
+                                                      (float*)L.e2, L.h, c->cc1.data(), c->cc2.data()));
   }
   e = (float*)L.e2;
   return GBMG_OK;
