@@ -39,7 +39,7 @@ __device__ __forceinline__ int problem_of(const I* __restrict__ off, int count, 
 }
 
 template <int V>
-__global__ void __maxnreg__(65536 / ((legs::DownTile<V>::T::NT + 127) / 128 * 128) / 8 * 8)
+__global__ void __maxnreg__(legs::max_regs<typename legs::DownTile<V>::T>())
 k_batch_down(BDesc B, Phases T, int l, legs::Coef cf) {
   using TL = typename legs::DownTile<V>::T;
   extern __shared__ __align__(16) float smf[];
@@ -63,7 +63,7 @@ k_batch_down(BDesc B, Phases T, int l, legs::Coef cf) {
 }
 
 template <int V>
-__global__ void __maxnreg__(65536 / ((legs::UpTile<V>::T::NT + 127) / 128 * 128) / 8 * 8)
+__global__ void __maxnreg__(legs::max_regs<typename legs::UpTile<V>::T>())
 k_batch_up(BDesc B, Phases T, int l, legs::Coef cf) {
   using TL = typename legs::UpTile<V>::T;
   extern __shared__ __align__(16) float smf[];

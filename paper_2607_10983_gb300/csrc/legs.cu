@@ -37,7 +37,7 @@ namespace {
 using namespace legs;
 
 template <int V, class TL>
-__global__ void __maxnreg__(65536 / ((TL::NT + 127) / 128 * 128) / 8 * 8)
+__global__ void __maxnreg__(max_regs<TL>())
 k_down_fused(Dims d, const float* __restrict__ r, float* __restrict__ e_out, float* __restrict__ rc, Sched sc,
              float inv_h2, Coef cf) {
   extern __shared__ float sm[];
@@ -57,7 +57,7 @@ k_down_fused(Dims d, const float* __restrict__ r, float* __restrict__ e_out, flo
 }
 
 template <int V, class TL>
-__global__ void __maxnreg__(65536 / ((TL::NT + 127) / 128 * 128) / 8 * 8)
+__global__ void __maxnreg__(max_regs<TL>())
 k_up_fused(Dims d, const float* __restrict__ e_in, const float* __restrict__ ec, const float* __restrict__ r,
            float* __restrict__ e_out, Sched sc, float inv_h2, Coef cf) {
   extern __shared__ float sm[];

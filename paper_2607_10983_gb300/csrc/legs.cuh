@@ -546,18 +546,25 @@ __device__ __forceinline__ void up_segment(Dims d, const float* __restrict__ e_i
 // (registers are granted to groups of four warps).  Down leg (degrees 1-3): columns of
 // R = 3 pairs, 512 threads, 16 warps per SM within 128 registers (0.450 ms at 512^3
 // against 0.468 with 4-pair columns in 384 threads and 0.484 with 6-pair columns in 256);
-// degree 4 (halo 5) keeps 4-pair columns, 384 threads and a 64 x 24 tile, which fit its
-// shared memory.  Up leg: columns of R = 4 pairs, 384 threads (even R makes each row's y
+// degree 4, whose five stages do not fit 168 registers, 5-pair columns of a 64 x 20 tile in 256
+// threads (up leg 4-pair): 256^3 0.155 -> 0.107 ms down, 0.174 -> 0.104 up against 384 threads
+// with 48 and 160 bytes of spill.  Up leg: columns of R = 4 pairs, 384 threads (even R makes each row's y
 // parity, and with it the prolongation's coarse-row pattern, a compile-time constant;
 // 6-pair columns in 256 threads 0.552 against 0.539 ms).
 template <int V>
 struct DownTile {
-  using T = typename std::conditional<(V >= 4), PTile<64, 24, V + 1, 384, 4>, PTile<64, 32, V + 1, 512, 3>>::type;
+  using T = typename std::conditional<(V >= 4), PTile<64, 20, V + 1, 256, 5>, PTile<64, 32, V + 1, 512, 3>>::type;
 };
 template <int V>
 struct UpTile {
-  using T = PTile<64, 32, V, 384, 4>;
+  using T = typename std::conditional<(V >= 4), PTile<64, 20, V, 256, 4>, PTile<64, 32, V, 384, 4>>::type;
 };
+// register limit of one CTA per SM (registers are granted to groups of four warps)
+template <class TL>
+constexpr int max_regs() {
+  constexpr int n = 65536 / ((TL::NT + 127) / 128 * 128) / 8 * 8;
+  return n < 255 ? n : 255;
+}
 
 template <int V>
 size_t down_smem() {
