@@ -106,10 +106,22 @@ __global__ void k_jacobi(Dims d, const T* __restrict__ r, const T* __restrict__ 
   e_out[i] = jacobi_step(c, r[i], nsum(load_nbrs(e_in, d, x, y, z, i), c), wa, wb);
 }
 
+// The first smoothing step of the level restricted to, from a zero iterate: e = d = a r (the
+// step's operations on zeros leave a r), in place of clearing e and a launch.
+template <typename T>
+struct FirstStep {
+  T *e, *d, a;
+  __device__ __forceinline__ void put(long long i, T r) const {
+    if (!e) return;
+    e[i] = t_mul(a, r);
+    if (d) d[i] = e[i];
+  }
+};
+
 // Full weighting, one thread per coarse cell: z-axis weights first, then y, then x
 // (the order the fused kernels use; ZS: the z weights as fw3z).
 template <typename T, bool ZS>
-__global__ void k_restrict(Dims df, const T* __restrict__ f, T* __restrict__ c) {
+__global__ void k_restrict(Dims df, const T* __restrict__ f, T* __restrict__ c, FirstStep<T> fs) {
   const Dims dc{df.nx / 2, df.ny / 2, df.nz / 2};
   const int X = blockIdx.x * BX + threadIdx.x, Y = blockIdx.y * BY + threadIdx.y, Z = blockIdx.z;
   if (X >= dc.nx || Y >= dc.ny) return;
@@ -133,7 +145,54 @@ __global__ void k_restrict(Dims df, const T* __restrict__ f, T* __restrict__ c) 
     }
     yv[a] = fw3(zv[0], zv[1], zv[2]);
   }
-  c[lin(dc, X, Y, Z)] = fw3(yv[0], yv[1], yv[2]);
+  const long long i = lin(dc, X, Y, Z);
+  const T v = fw3(yv[0], yv[1], yv[2]);
+  c[i] = v;
+  fs.put(i, v);
+}
+
+// Residual and full weighting of a small level in one launch, 4 x 4 x 2 coarse cells per CTA:
+// a thread computes the residual of one of the 9 x 9 x 5 fine cells under them, then the z, y
+// and x weights in turn.  The two launches, the second with 27 loads and 39 operations per coarse
+// cell in a few CTAs, are latency-bound, and FP64 (two operations per clock and SM) wants every
+// SM: 32^3 6.3 -> 3.0 us, 48^3 8.0 -> 5.3 (FP32 3.1 -> 1.9, 3.6 -> 2.6).  From 64^3 on the halo's
+// repeated residuals cost more (11.0 against 9.6 us).
+constexpr int RX = 9, RZ = 5, RNT = 416;   // fine cells per side (x, y), in z; threads
+template <typename T>
+__global__ void __launch_bounds__(RNT) k_residual_restrict(Dims df, const T* __restrict__ f, const T* __restrict__ u,
+                                                           T inv_h2, T* __restrict__ c, FirstStep<T> fs) {
+  __shared__ T r[RZ][RX][RX], zw[2][RX][RX], yw[2][4][RX];
+  const Dims dc{df.nx / 2, df.ny / 2, df.nz / 2};
+  const int t = threadIdx.x, X0 = 4 * blockIdx.x, Y0 = 4 * blockIdx.y, Z0 = 2 * blockIdx.z;
+  // sides of at least 8 cells: a tile reaches at most 6 cells over the end
+  auto wrap = [](int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); };
+  if (t < RX * RX * RZ) {
+    const int x = t % RX, y = t / RX % RX, z = t / (RX * RX);
+    const int gx = wrap(2 * X0 - 1 + x, df.nx), gy = wrap(2 * Y0 - 1 + y, df.ny), gz = wrap(2 * Z0 - 1 + z, df.nz);
+    const long long i = lin(df, gx, gy, gz);
+    r[z][y][x] = resid_from_sum(f[i], nsum(load_nbrs(u, df, gx, gy, gz, i), u[i]), inv_h2);
+  }
+  __syncthreads();
+  if (t < 2 * RX * RX) {
+    const int x = t % RX, y = t / RX % RX, z = t / (RX * RX);
+    const T a = r[2 * z][y][x], b = r[2 * z + 1][y][x], e = r[2 * z + 2][y][x];
+    if constexpr (sizeof(T) == 4) zw[z][y][x] = fw3z(a, b, e);
+    else zw[z][y][x] = fw3(a, b, e);
+  }
+  __syncthreads();
+  if (t < 2 * 4 * RX) {
+    const int x = t % RX, y = t / RX % 4, z = t / (4 * RX);
+    yw[z][y][x] = fw3(zw[z][2 * y][x], zw[z][2 * y + 1][x], zw[z][2 * y + 2][x]);
+  }
+  __syncthreads();
+  if (t < 32) {
+    const int x = t % 4, y = t / 4 % 4, z = t / 16;
+    if (X0 + x >= dc.nx || Y0 + y >= dc.ny || Z0 + z >= dc.nz) return;
+    const long long i = lin(dc, X0 + x, Y0 + y, Z0 + z);
+    const T v = fw3(yw[z][y][2 * x], yw[z][y][2 * x + 1], yw[z][y][2 * x + 2]);
+    c[i] = v;
+    fs.put(i, v);
+  }
 }
 
 template <typename T>
@@ -438,11 +497,19 @@ cudaError_t launch_jacobi(cudaStream_t st, Dims d, const T* r, const T* e_in, T*
   return cudaGetLastError();
 }
 template <typename T>
-cudaError_t launch_restrict(cudaStream_t st, Dims fine, const T* f, T* c, bool geometry) {
+cudaError_t launch_restrict(cudaStream_t st, Dims fine, const T* f, T* c, bool geometry, T* e, T* dv, T a) {
   const Dims dc{fine.nx / 2, fine.ny / 2, fine.nz / 2};
   constexpr bool zs = sizeof(T) == 4;
-  if (zs && !geometry) k_restrict<T, zs><<<cell_grid(dc), dim3(BX, BY), 0, st>>>(fine, f, c);
-  else k_restrict<T, false><<<cell_grid(dc), dim3(BX, BY), 0, st>>>(fine, f, c);
+  if (zs && !geometry) k_restrict<T, zs><<<cell_grid(dc), dim3(BX, BY), 0, st>>>(fine, f, c, FirstStep<T>{e, dv, a});
+  else k_restrict<T, false><<<cell_grid(dc), dim3(BX, BY), 0, st>>>(fine, f, c, FirstStep<T>{e, dv, a});
+  note_launch();
+  return cudaGetLastError();
+}
+template <typename T>
+cudaError_t launch_residual_restrict(cudaStream_t st, Dims fine, const T* f, const T* u, T inv_h2, T* c, T* e, T* dv,
+                                     T a) {
+  const dim3 g((fine.nx + 7) / 8, (fine.ny + 7) / 8, (fine.nz + 3) / 4);
+  k_residual_restrict<T><<<g, RNT, 0, st>>>(fine, f, u, inv_h2, c, FirstStep<T>{e, dv, a});
   note_launch();
   return cudaGetLastError();
 }
@@ -541,7 +608,8 @@ cudaError_t launch_df_update(cudaStream_t st, long long n, float2* phi, const fl
   template cudaError_t launch_residual<T>(cudaStream_t, Dims, const T*, const T*, T*, T, double*);   \
   template cudaError_t launch_cheb_step<T>(cudaStream_t, Dims, const T*, const T*, T*, T*, T, T, T);  \
   template cudaError_t launch_jacobi<T>(cudaStream_t, Dims, const T*, const T*, T*, T, T);           \
-  template cudaError_t launch_restrict<T>(cudaStream_t, Dims, const T*, T*, bool);                         \
+  template cudaError_t launch_restrict<T>(cudaStream_t, Dims, const T*, T*, bool, T*, T*, T);                         \
+  template cudaError_t launch_residual_restrict<T>(cudaStream_t, Dims, const T*, const T*, T, T*, T*, T*, T); \
   template cudaError_t launch_prolong_add<T>(cudaStream_t, Dims, const T*, T*);                      \
   template cudaError_t launch_coarse_matvec<T>(cudaStream_t, int, const T*, const T*, T*);           \
   template cudaError_t launch_sum<T>(cudaStream_t, long long, const T*, double*, double*);           \

@@ -35,7 +35,13 @@ inline void cheb_constants(double c2, double h, double& a, double& b) {
 }
 // geometry: a curvilinear level's coefficients (FP32 residuals add the z weights as fw3z)
 template <typename T>
-cudaError_t launch_restrict(cudaStream_t st, Dims fine, const T* f, T* c, bool geometry = false);
+cudaError_t launch_restrict(cudaStream_t st, Dims fine, const T* f, T* c, bool geometry = false, T* e = nullptr,
+                            T* dv = nullptr, T a = T(0));
+// c = restriction of f - A u; for both, e (nullable) = dv (nullable) = a c: the first smoothing
+// step of the coarse level from zero.
+template <typename T>
+cudaError_t launch_residual_restrict(cudaStream_t st, Dims fine, const T* f, const T* u, T inv_h2, T* c, T* e, T* dv,
+                                     T a);
 template <typename T>
 cudaError_t launch_prolong_add(cudaStream_t st, Dims coarse, const T* c, T* f);
 template <typename T>
