@@ -10,6 +10,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include "chain.cuh"
 #include "kernels.h"
 #include "stencil.cuh"
 
@@ -246,6 +247,37 @@ __global__ void k_coarse_matvec(int n, const T* __restrict__ G, const T* __restr
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc = t_add(acc, __shfl_xor_sync(0xffffffffu, acc, o));
   if (lane == 0) e[row] = acc;
+}
+
+// The FP64 chain's bottom: k_cheb_step, k_residual, k_restrict, k_prolong_add and
+// k_coarse_matvec of the levels from a small one down (chain.cuh).
+constexpr int kChainThreads = 256;   // one cell of 16^3 per thread
+struct ChainArgs64 {
+  chain::Fields<double> F;
+  ChainCheb k;
+};
+struct ChainOp64 {
+  using T = double;
+  static constexpr int kDone = 1;
+  const ChainArgs64& A;
+  __device__ __forceinline__ const chain::Fields<double>& f() const { return A.F; }
+  __device__ __forceinline__ double step(int l, int k, const chain::View<double>& u, double e, double r, double& dv,
+                                         int i, const chain::Cell& c) const {
+    const Dims d = A.F.lv[l].d;
+    const int pl = d.nx * d.ny;
+    const double xm = u[i + (c.x == 0 ? d.nx - 1 : -1)], xp = u[i + (c.x == d.nx - 1 ? 1 - d.nx : 1)];
+    const double ym = u[i + (c.y == 0 ? d.ny - 1 : -1) * d.nx], yp = u[i + (c.y == d.ny - 1 ? 1 - d.ny : 1) * d.nx];
+    const double zm = u[i + (c.z == 0 ? d.nz - 1 : -1) * pl], zp = u[i + (c.z == d.nz - 1 ? 1 - d.nz : 1) * pl];
+    const double s = lap_sum(xm, xp, ym, yp, zm, zp, e);
+    if (k < 0) return resid_from_sum(r, s, A.k.ih2[l]);
+    return cheb_step(e, r, s, dv, A.k.a[l][k], A.k.b[l][k], A.k.c1[k]);
+  }
+  __device__ __forceinline__ double first(int l, double r, double& dv, int) const {
+    return dv = t_mul(A.k.a[l][0], r);
+  }
+};
+__global__ void __launch_bounds__(kChainThreads) k_chain_f64(const __grid_constant__ ChainArgs64 A) {
+  chain::run(ChainOp64{A});
 }
 
 template <typename T>
@@ -512,6 +544,10 @@ cudaError_t launch_residual_restrict(cudaStream_t st, Dims fine, const T* f, con
   k_residual_restrict<T><<<g, RNT, 0, st>>>(fine, f, u, inv_h2, c, FirstStep<T>{e, dv, a});
   note_launch();
   return cudaGetLastError();
+}
+cudaError_t launch_chain_f64(cudaStream_t st, chain::Fields<double> f, const ChainCheb& k) {
+  const size_t smem = chain::layout(f);
+  return chain::launch(st, k_chain_f64, kChainThreads, smem, ChainArgs64{f, k});
 }
 template <typename T>
 cudaError_t launch_prolong_add(cudaStream_t st, Dims coarse, const T* c, T* f) {

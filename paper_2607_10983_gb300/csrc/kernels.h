@@ -27,6 +27,16 @@ cudaError_t launch_cheb_step(cudaStream_t st, Dims d, const T* r, const T* e_in,
 // Weighted Jacobi with wa = omega D^-1, wb = wa / h^2.
 template <typename T>
 cudaError_t launch_jacobi(cudaStream_t st, Dims d, const T* r, const T* e_in, T* e_out, T wa, T wb);
+// One launch for the bottom of a V-cycle (chain.cuh): the top level's e (and d) hold its first
+// smoothing step, and e receives the result.
+namespace chain {
+template <typename T>
+struct Fields;
+}
+struct ChainCheb {   // FP64: constants per level and step
+  double a[8][8], b[8][8], c1[8], ih2[8];
+};
+cudaError_t launch_chain_f64(cudaStream_t st, chain::Fields<double> f, const ChainCheb& k);
 // Folded Chebyshev constants of step k on a level of spacing h.
 inline void cheb_constants(double c2, double h, double& a, double& b) {
   const double dinv = -(h * h) / 6.0;

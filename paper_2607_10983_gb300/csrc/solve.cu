@@ -4,6 +4,7 @@
 #include <cstring>
 #include <vector>
 
+#include "chain.cuh"
 #include "kernels.h"
 #include "loop.h"
 #include "solver.h"
@@ -91,6 +92,35 @@ gbmg_status store_coarse_correction(gbmg_ctx* c, int l, float* e) {
   return GBMG_OK;
 }
 
+// FP64 Chebyshev levels of at most this many cells, with at least one smoothed level, run in
+// one launch from the first step on.
+constexpr long long kChainCells64 = 4096;
+bool chain64_from(const gbmg_ctx* c, int l) {
+  return c->o.smoother == GBMG_SMOOTH_CHEBYSHEV && c->o.degree >= 1 && c->o.degree <= 8 && l >= 1 && c->L - l >= 2 &&
+         c->L - l <= chain::kMaxL && ncell(c->lv[l].d) <= kChainCells64;
+}
+gbmg_status chain64(gbmg_ctx* c, int l0, double*& e) {
+  chain::Fields<double> F{};
+  ChainCheb K{};
+  F.nl = c->L - l0;
+  F.pre = c->o.degree - 1;
+  F.post = c->o.degree;
+  F.nc = c->nc;
+  F.G = c->G64;
+  for (int k = 0; k < c->o.degree; ++k) K.c1[k] = c->cc1[k];
+  for (int i = 0; i < F.nl; ++i) {
+    const Level& L = c->lv[l0 + i];
+    F.lv[i].d = L.d;
+    K.ih2[i] = 1.0 / (L.h * L.h);
+    for (int k = 0; k < c->o.degree; ++k) cheb_constants(c->cc2[k], L.h, K.a[i][k], K.b[i][k]);
+  }
+  e = F.e = (double*)c->lv[l0].e;
+  F.r = (double*)c->lv[l0].r;
+  F.d = (double*)c->lv[l0].dv;
+  TRY(launch_chain_f64(c->stream, F, K));
+  return GBMG_OK;
+}
+
 // Levels below this size run residual and restriction as one launch (48^3 in FP64: 5.3 against
 // 8.0 us; 64^3: 11.0 against 9.6).
 constexpr long long kResRestrictCells = 1ll << 18;
@@ -111,6 +141,9 @@ gbmg_status vcycle_unfused(gbmg_ctx* c, int l, T*& e, T*& eo, const T* r, int do
       TRY(launch_small_vcycle(c->stream, P, r, e));
       return GBMG_OK;
     }
+  }
+  if constexpr (sizeof(T) == 8) {
+    if (done == 1 && chain64_from(c, l)) return chain64(c, l, e);
   }
   T* dv = (T*)L.dv;
   TRYS(smooth_pass<T>(c, l, e, eo, r, dv, false, done));
