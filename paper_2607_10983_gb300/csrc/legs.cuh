@@ -99,6 +99,13 @@ __device__ __forceinline__ int tile_phase(long long u0, int nz, long long total,
 __device__ __forceinline__ float2 ld2(const float* p) { return __ldg(reinterpret_cast<const float2*>(p)); }
 __device__ __forceinline__ void st2(float* p, float2 v) { *reinterpret_cast<float2*>(p) = v; }
 
+// f(0), .., f(V - 1) with constant arguments
+template <int V, class F>
+__device__ __forceinline__ void warm_up(F f) {
+  if constexpr (V > 1) warm_up<V - 1>(f);
+  f(std::integral_constant<int, V - 1>());
+}
+
 // ------------------------------------------------------------------ down leg
 //
 // Addressing.  Every shared access of a thread is a compile-time offset from one of two
@@ -119,7 +126,12 @@ __device__ __forceinline__ void st2(float* p, float2 v) { *reinterpret_cast<floa
 // came before the barrier (0.58 ms).  A few bytes of spill cost more than all of this gives
 // (up leg 0.95 ms at 40 bytes): the L1 beside the shared planes is small.
 // 512^3, degree 3: down 0.531 -> 0.445 ms, up 0.658 -> 0.539; 64^3: 14.5 -> 12.5 us each.
-// Prefetching planes to L2 two ahead: 0.471 ms down.
+// Prefetching planes to L2 two ahead: 0.471 ms down; staging r by asynchronous copies three
+// planes ahead: 0.464.
+// The first 2 V planes of a down segment feed only the stages that a plane of the segment will
+// depend on, in code of their own (short segments, of small meshes, are mostly such planes:
+// 64^3 12.4 -> 10.4 us, 256^3 73.6 -> 69.1; 512^3 0.445 -> 0.450 ms).  The same in the up leg
+// spills (24 bytes, 512^3 0.539 -> 0.555 ms; behind branches in the loop 0.92).
 
 template <int V, class TL>
 __device__ __forceinline__ void down_segment(Dims d, const float* __restrict__ r, float* __restrict__ e_out,
@@ -163,16 +175,18 @@ __device__ __forceinline__ void down_segment(Dims d, const float* __restrict__ r
     for (int s = 0; s < V + 2; ++s) wt[s][j] = Z, wc[s][j] = Z;
     zwp[j] = Z;
   }
-  // the last coarse plane c = zend - 1 (a segment may end on an odd plane) is
+  // the last coarse plane, c = zend - 2 or zend - 1 (a segment may end on an odd plane), is
   // written at t = c + V + 2
-  const int tb = z0 - H, te = zend + V + 1;
+  const int tb = z0 - H, te = zend + V + (zend & 1);
   int zl = wrapmod(tb, d.nz);                   // plane of the latest load of r
   const float* rl = r + (size_t)zl * pst;
 #pragma unroll
   for (int j = 0; j < R; ++j) rnext[j] = ld2(rl + P.goff[j]);
-  // one plane; CUR: its buffer (t - tb) & 1, a constant
-  auto step = [&](int t, auto CUR) {
+  // one plane; CUR: its buffer (t - tb) & 1, a constant; ACT: stages 2 .. ACT + 1 run, and with
+  // ACT = V the residual and the coarse output
+  auto step = [&](int t, auto CUR, auto ACT) {
     const int cur = CUR;
+    constexpr int act = decltype(ACT)::value;
     float* const bc = bs + (cur ? PLANE : 0);
     const float* const bp = bs + (cur ? 0 : PLANE);
 #pragma unroll
@@ -202,6 +216,11 @@ __device__ __forceinline__ void down_segment(Dims d, const float* __restrict__ r
     // stages 2..V: Chebyshev steps with the stencil on e_{s-1}
 #pragma unroll
     for (int s = 2; s <= V; ++s) {
+      if (s > act + 1) {
+#pragma unroll
+        for (int j = 0; j < R; ++j) en[s][j] = dn[s][j] = Z;
+        continue;
+      }
       const float* const sE = bp + (s - 2) * SP;
       float* const dE = bc + (s - 1) * SP;
 #pragma unroll
@@ -229,7 +248,7 @@ __device__ __forceinline__ void down_segment(Dims d, const float* __restrict__ r
     }
     // residual stage at plane c + 1 = t - V; on odd planes the z weights of the restriction
     // at c
-    {
+    if (act == V) {
       const float* const sE = bp + (V - 1) * SP;
       float* const zE = bc + V * SP;
       const int c = t - V - 1;
@@ -259,7 +278,7 @@ __device__ __forceinline__ void down_segment(Dims d, const float* __restrict__ r
     // coarse output from the z-weighted plane of the previous iteration: y weights
     // for the x offsets -1, 0, +1 (odd cell of the pair to the left, even and odd
     // cell of the centre pair), then x weights
-    {
+    if (act == V) {
       const int c = t - V - 2;
       if (((c & 1) == 0) && c >= z0 && c < zend) {
         const float* const zE = sm + PAD + V * SP + (cur ? 0 : PLANE);
@@ -289,10 +308,14 @@ __device__ __forceinline__ void down_segment(Dims d, const float* __restrict__ r
     }
     __syncthreads();
   };
-  for (int t = tb;; t += 2) {
-    step(t, std::integral_constant<int, 0>());
+  warm_up<V>([&](auto K) {
+    step(tb + 2 * K, std::integral_constant<int, 0>(), K);
+    step(tb + 2 * K + 1, std::integral_constant<int, 1>(), K);
+  });
+  for (int t = tb + 2 * V;; t += 2) {
+    step(t, std::integral_constant<int, 0>(), std::integral_constant<int, V>());
     if (t == te) break;
-    step(t + 1, std::integral_constant<int, 1>());
+    step(t + 1, std::integral_constant<int, 1>(), std::integral_constant<int, V>());
     if (t + 1 == te) break;
   }
 }
