@@ -1261,10 +1261,12 @@ long long curv_df_partials(Dims d, int form) {
   return (long long)g.x * g.y * g.z;
 }
 
-// FP32 sweeps and residuals of levels of at most 32^3 cells run one thread per cell
+// FP32 sweeps and residuals of levels of at most 64^3 cells run one thread per cell
 // (k_curv_jacobi / k_curv_residual: every load of a cell in one round) instead of the
-// marching tiles, whose few CTAs there take one dependent round of loads per plane.
-static bool curv_cellwise(Dims d) { return (long long)d.nx * d.ny * d.nz <= 32 * 32 * 32; }
+// marching tiles, whose few CTAs there take one dependent round of loads per plane: a sweep
+// of M 2.9 us at 32^3, 4.8 against 6.9 at 56^3, 5.6 against 6.5 at 64^3 (M^T 4.9 against 7.1 and S
+// 5.1 against 7.0 at 56^3); at 80 x 64 x 96 the tiles' 9.2 us is where the cells' would be.
+static bool curv_cellwise(Dims d) { return (long long)d.nx * d.ny * d.nz <= 64 * 64 * 64; }
 
 cudaError_t launch_curv_diag(cudaStream_t st, Dims d, const CurvCoef& cf, int form, float* D) {
   k_curv_diag<<<cell_grid(d), dim3(BX, BY), 0, st>>>(d, cf, form, D);

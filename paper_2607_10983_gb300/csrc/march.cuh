@@ -127,15 +127,16 @@ struct View {
   }
 };
 
-// z planes per CTA: among runs of 4 .. nz planes the one with the least work on the
-// critical path, whole waves of `resident` CTAs times the run plus its two extra planes.
+// z planes per CTA: among runs of 2 .. nz planes the one with the least work on the
+// critical path, whole waves of `resident` CTAs times the run plus its two extra planes (from 4
+// planes on: a sweep of 80 x 64 x 96 9.5 instead of 9.2 us, of 64^3 7.4 instead of 6.7).
 inline int march_zchunk(Dims d, int resident) {
   const long long tiles = (long long)((d.nx + MX - 1) / MX) * ((d.ny + MY - 1) / MY);
   int best = d.nz;
   long long best_cost = -1;
   for (int n = 1; n <= d.nz; ++n) {
     const int zc = (d.nz + n - 1) / n;
-    if (zc < 4 && n > 1) break;
+    if (zc < 2 && n > 1) break;
     const long long waves = (tiles * ((d.nz + zc - 1) / zc) + resident - 1) / resident;
     const long long cost = waves * (zc + 2);
     if (best_cost < 0 || cost < best_cost) best_cost = cost, best = zc;

@@ -12,7 +12,8 @@ torch = pytest.importorskip("torch")
 
 
 @pytest.mark.parametrize("sym", [False, True])
-@pytest.mark.parametrize("shape", [(48, 40, 56), (80, 64, 40), (32, 40, 96), (40, 96, 64), (112, 32, 32)])
+@pytest.mark.parametrize("shape", [(48, 40, 56), (80, 64, 40), (32, 40, 96), (40, 96, 64), (112, 32, 32),
+                                   (64, 64, 80), (80, 112, 64), (64, 96, 112)])
 def test_march_equals_tiles(gb, shape, sym):
     s = gb.Solver(shape, op="curv", curv_sym=sym)
     s.set_geometry(torch.from_numpy(smoothed_grf(shape, 81, 2.0, 0.5)).cuda())
