@@ -125,13 +125,13 @@ void mg_destroy(gbmg_ctx* ctx);
 /* Queue later work on `cuda_stream` (a cudaStream_t; NULL = legacy default stream). */
 gbmg_status mg_set_stream(gbmg_ctx* ctx, void* cuda_stream);
 
-/* Cycle graphs (default on).  A mixed fused flat solve (V-cycle or krylov corrections)
- * and a curvilinear solve run each V-cycle of the defect correction (Sec. 3.2) as one
- * CUDA graph launch: the cycle's launches are captured once per context (per buffer
- * parity or orientation, after one cycle has run eagerly) and replayed; the host still
- * checks convergence after every cycle.  Results are the same bits either way.
- * enable = 0 launches every kernel of every cycle from the host.  Timed kernel families
- * (mg_profile_begin) are timed inside the graphs by event nodes. */
+/* Cycle graphs (default on).  FP64 flat solves, mixed fused flat solves (V-cycle or krylov
+ * corrections) and curvilinear solves run the V-cycles of the defect correction (Sec. 3.2)
+ * as one CUDA graph that loops on the device: it is captured once per context (and
+ * orientation) and launched once per solve, and the host waits once.  While kernel families
+ * are timed (mg_profile_begin), each cycle of a mixed solve is a graph launch of its own
+ * with event nodes, and the host checks convergence after every cycle.  Results are the
+ * same bits either way.  enable = 0 launches every kernel of every cycle from the host. */
 gbmg_status mg_set_cycle_graphs(gbmg_ctx* ctx, int enable);
 
 /* Curvilinear contexts only: set the deformation potential psi (nx*ny*nz doubles,

@@ -16,6 +16,9 @@
 // per problem over fixed chunks in a fixed order (deterministic).  A problem that has
 // converged (or failed) skips its work; the loop ends when none is active or
 // max_vcycles is reached.  Per-problem completion times come from %globaltimer.
+//
+// With mg_batch_use_graph the phases run as kernels of a graph instead where every level is
+// fused or in a bottom cycle (batch_graph.cu): 48 problems 13.0 ms launched here, 8.2 there.
 #include <cooperative_groups.h>
 
 #include <algorithm>

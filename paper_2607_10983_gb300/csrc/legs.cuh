@@ -2,7 +2,7 @@
 // geometry, per-thread pair columns and one z segment of the down leg (Chebyshev
 // pre-smoothing from zero, residual, full-weighting restriction) and of the up leg
 // (trilinear prolongation + correction, Chebyshev post-smoothing).  Used by the
-// per-level kernels of legs.cu and by the batched persistent kernel.
+// per-level kernels of legs.cu, the batched persistent kernel and the batches' phase graph.
 #pragma once
 #include <type_traits>
 
