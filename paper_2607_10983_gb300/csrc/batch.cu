@@ -832,7 +832,11 @@ extern "C" gbmg_status mg_batch_create(gbmg_batch** out, gbmg_ctx* const* ctxs, 
     }
   }
   gbmg_status st = build_tables(b);
-  if (st == GBMG_OK) st = b->phases.init(b->ctx, b->hprob, D, bottom);
+  if (st == GBMG_OK && b->phases.init(b->ctx, b->hprob, D, bottom) != GBMG_OK) {
+    b->phases.usable = false;  // the persistent kernel needs nothing more
+    (void)cudaGetLastError();
+    g_last_error.clear();
+  }
   // persistent grid: every block resident at once (cooperative launch)
   if (st == GBMG_OK) st = max_blocks(b, b->blocks);
   if (st != GBMG_OK) {
@@ -926,14 +930,17 @@ extern "C" gbmg_status mg_batch_solve(gbmg_batch* b, const double* const* src_de
         b->gexec = nullptr;
       }
       cudaGraph_t graph = nullptr;
-      if (b->phases.usable) {
-        const gbmg_status cs = b->phases.build(b->gstream, D, &graph, [&]() { return copy_in(b->gstream); },
-                                               [&]() { return copy_out(b->gstream); });
-        if (cs != GBMG_OK) {
-          if (graph) cudaGraphDestroy(graph);
-          return cs;
-        }
-      } else {
+      // (an incomplete phase graph, say on a driver without conditional nodes, leaves the
+      // batch on the persistent kernel)
+      if (b->phases.usable && b->phases.build(b->gstream, D, &graph, [&]() { return copy_in(b->gstream); },
+                                              [&]() { return copy_out(b->gstream); }) != GBMG_OK) {
+        if (graph) cudaGraphDestroy(graph);
+        graph = nullptr;
+        b->phases.usable = false;
+        (void)cudaGetLastError();
+        g_last_error.clear();
+      }
+      if (!b->phases.usable) {
         TRY(cudaStreamBeginCapture(b->gstream, cudaStreamCaptureModeThreadLocal));
         const gbmg_status cs = enqueue(b->gstream);
         const cudaError_t ce = cudaStreamEndCapture(b->gstream, &graph);
