@@ -372,6 +372,52 @@ __global__ void k_curv_restrict(Dims df, const float* __restrict__ f, float* __r
   }
 }
 
+// k_curv_residual and k_curv_restrict of a small level in one launch, 4 x 4 x 2 coarse cells per
+// CTA (the form of k_residual_restrict of the flat path): a thread computes the residual of one
+// of the 9 x 9 x 5 fine cells under them, then the z, y and x weights in turn; the same
+// operations per cell.  The two launches are bound by latency: 16^3 4.3 -> 3.6 us, 40 x 32 x 48
+// 5.9 -> 5.1, and a gap between graph nodes less; the halo's repeated residuals (1.6 per cell) limit
+// it to 64 x 32 x 32 cells (32^3 4.9 us both ways).
+constexpr int RX = 9, RZ = 5, RNT = 416;   // fine cells per side (x, y), in z; threads
+__global__ void __launch_bounds__(RNT) k_curv_residual_restrict(Dims df, CurvCoef cf, const float* __restrict__ r,
+                                                                const float* __restrict__ u, float inv_h2, int form,
+                                                                float* __restrict__ rc, float* __restrict__ e1,
+                                                                const float* __restrict__ J,
+                                                                const float* __restrict__ D, float h2, float omega) {
+  __shared__ float t[RZ][RX][RX], zw[2][RX][RX], yw[2][4][RX];
+  const Dims dc{df.nx / 2, df.ny / 2, df.nz / 2};
+  const int q = threadIdx.x, X0 = 4 * blockIdx.x, Y0 = 4 * blockIdx.y, Z0 = 2 * blockIdx.z;
+  // sides of at least 8 cells: a tile reaches at most 6 cells over the end
+  auto wrap = [](int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); };
+  if (q < RX * RX * RZ) {
+    const int x = q % RX, y = q / RX % RX, z = q / (RX * RX);
+    const Nbhd nb(df, wrap(2 * X0 - 1 + x, df.nx), wrap(2 * Y0 - 1 + y, df.ny), wrap(2 * Z0 - 1 + z, df.nz));
+    const FieldAt<float> U{u, &nb};
+    const CoefAt Bc{cf, &nb};
+    const long long i = nb(0, 0, 0);
+    t[z][y][x] = r[i] - op_h2<float>(U, Bc, form) * inv_h2 / cf.J[i];
+  }
+  __syncthreads();
+  if (q < 2 * RX * RX) {
+    const int x = q % RX, y = q / RX % RX, z = q / (RX * RX);
+    zw[z][y][x] = fw3(t[2 * z][y][x], t[2 * z + 1][y][x], t[2 * z + 2][y][x]);
+  }
+  __syncthreads();
+  if (q < 2 * 4 * RX) {
+    const int x = q % RX, y = q / RX % 4, z = q / (4 * RX);
+    yw[z][y][x] = fw3(zw[z][2 * y][x], zw[z][2 * y + 1][x], zw[z][2 * y + 2][x]);
+  }
+  __syncthreads();
+  if (q < 32) {
+    const int x = q % 4, y = q / 4 % 4, z = q / 16;
+    if (X0 + x >= dc.nx || Y0 + y >= dc.ny || Z0 + z >= dc.nz) return;
+    const long long i = lin(dc, X0 + x, Y0 + y, Z0 + z);
+    const float v = fw3(yw[z][y][2 * x], yw[z][y][2 * x + 1], yw[z][y][2 * x + 2]);
+    rc[i] = v;
+    if (e1) e1[i] = jacobi_value(0.f, v, J[i], D[i], 0.f, h2, omega);
+  }
+}
+
 // Dense matrix of the level operator (row-major n x n, FP64): entry (i, j) = (op(e_j) / J)_i.
 struct UnitAt {
   const Nbhd* nb;
@@ -1328,6 +1374,19 @@ cudaError_t launch_curv_restrict(cudaStream_t st, Dims fine, const float* f, flo
   while (zc > 1 && cols * ((dc.nz + zc - 1) / zc) < 4 * 152) zc /= 2;
   k_curv_restrict<<<dim3((dc.nx + BX - 1) / BX, (dc.ny + BY - 1) / BY, (dc.nz + zc - 1) / zc), dim3(BX, BY), 0, st>>>(
       fine, f, rc, e1, cc.J, cc.D, cc.h2, omega, zc);
+  note_launch();
+  return cudaGetLastError();
+}
+
+bool curv_residual_restrict_ok(Dims d) {
+  return ncell(d) <= 64 * 32 * 32 && d.nx >= 8 && d.ny >= 8 && d.nz >= 8;
+}
+cudaError_t launch_curv_residual_restrict(cudaStream_t st, Dims fine, const CurvCoef& cf, const float* r, const float* u,
+                                          int form, float* rc, const CurvCoef& cc, float* e1, float omega) {
+  if (form < 0 || form > 2) return cudaErrorInvalidValue;
+  const dim3 g((fine.nx + 7) / 8, (fine.ny + 7) / 8, (fine.nz + 3) / 4);
+  k_curv_residual_restrict<<<g, RNT, 0, st>>>(fine, cf, r, u, (float)(1.0 / cf.h2), form, rc, e1, cc.J, cc.D, cc.h2,
+                                              omega);
   note_launch();
   return cudaGetLastError();
 }

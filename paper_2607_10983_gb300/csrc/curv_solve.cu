@@ -47,13 +47,18 @@ gbmg_status vcycle_curv(gbmg_ctx* c, int l, float*& e, float*& eo, const float* 
     return GBMG_OK;
   }
   TRYS(curv_smooth(c, l, e, eo, r, c->o.nu1 - 1, tr));
-  TRY(launch_curv_residual(c->stream, L.d, L.cc, r, e, (float*)L.t, curv_form(c, tr)));
   const Level& C = c->lv[l + 1];
   float* ce = (float*)C.e;
   float* ceo = (float*)C.e2;
   const bool smoothed = l + 1 < c->L - 1;
-  TRY(launch_curv_restrict(c->stream, L.d, (const float*)L.t, (float*)C.r, C.cc, smoothed && c->o.nu1 > 0 ? ce : nullptr,
-                           (float)c->o.omega));
+  float* const first = smoothed && c->o.nu1 > 0 ? ce : nullptr;
+  if (curv_residual_restrict_ok(L.d)) {
+    TRY(launch_curv_residual_restrict(c->stream, L.d, L.cc, r, e, curv_form(c, tr), (float*)C.r, C.cc, first,
+                                      (float)c->o.omega));
+  } else {
+    TRY(launch_curv_residual(c->stream, L.d, L.cc, r, e, (float*)L.t, curv_form(c, tr)));
+    TRY(launch_curv_restrict(c->stream, L.d, (const float*)L.t, (float*)C.r, C.cc, first, (float)c->o.omega));
+  }
   if (smoothed && c->o.nu1 == 0) TRY(cudaMemsetAsync(ce, 0, (size_t)ncell(C.d) * sizeof(float), c->stream));
   TRYS(vcycle_curv(c, l + 1, ce, ceo, (const float*)C.r, tr));
   TRY(launch_prolong_add<float>(c->stream, C.d, ce, e));

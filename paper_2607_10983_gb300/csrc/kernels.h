@@ -172,6 +172,10 @@ cudaError_t launch_march_jacobi(cudaStream_t st, Dims d, const CurvCoef& cf, con
 cudaError_t launch_march_residual(cudaStream_t st, Dims d, const CurvCoef& cf, const float* r, const float* u,
                                   float* out, int form);
 // dense n x n matrix of op / J on a (small) level, FP64 row-major
+// Both steps of a small level's down leg (launch_curv_residual, launch_curv_restrict) in one launch.
+bool curv_residual_restrict_ok(Dims d);
+cudaError_t launch_curv_residual_restrict(cudaStream_t st, Dims fine, const CurvCoef& cf, const float* r, const float* u,
+                                          int form, float* rc, const CurvCoef& cc, float* e1, float omega);
 cudaError_t launch_curv_dense(cudaStream_t st, Dims d, CurvCoef cf, int form, double* out);
 // Minimum-norm inverses (dense_pinv) of two dense n x n FP64 operators (the coarsest
 // operator and its transposed-solve twin, dense) with left null vector J, n <= 512, in FP64
