@@ -325,50 +325,57 @@ __global__ void k_curv_jacobi_zero(long long n, const float* __restrict__ J, con
 // Full weighting to a coarse level and the first sweep of its pre-smoothing, from zero: one
 // thread per coarse column of zc planes.  The weights run along z first, then y, then x
 // (k_restrict's order and bits); a thread reads each fine plane once, as one x-pair and one
-// odd cell per row, 12 loads per coarse cell instead of 27.  256^3: 35 -> 18 us, and the
-// sweep's own pass over r, J and D is gone.
+// odd cell per row, 12 loads per coarse cell instead of 27, and the next coarse cell's planes
+// are loaded before the current one is formed (latency bounds it: 256^3 35.0 -> 24.7 us after
+// a cold L1, 128^3 9.7 -> 7.8).
+constexpr int RBY = 4;   // rows of a CTA
 __global__ void k_curv_restrict(Dims df, const float* __restrict__ f, float* __restrict__ rc, float* __restrict__ e1,
                                 const float* __restrict__ J, const float* __restrict__ D, float h2, float omega, int zc) {
   const Dims dc{df.nx / 2, df.ny / 2, df.nz / 2};
-  const int X = blockIdx.x * BX + threadIdx.x, Y = blockIdx.y * BY + threadIdx.y;
+  const int X = blockIdx.x * BX + threadIdx.x, Y = blockIdx.y * RBY + threadIdx.y;
   if (X >= dc.nx || Y >= dc.ny) return;
   const int Z0 = blockIdx.z * zc, Z1 = min(Z0 + zc, dc.nz);
   const long long pst = (long long)df.nx * df.ny;
   int row[3];
 #pragma unroll
-  for (int k = 0; k < 3; ++k) row[k] = wrapi(2 * Y + k - 1, df.ny) * df.nx;
-  const int xm = wrapi(2 * X - 1, df.nx);
+  for (int k = 0; k < 3; ++k) row[k] = wrapi(2 * Y + k - 1, df.ny) * df.nx + 2 * X;
+  const int xm = wrapi(2 * X - 1, df.nx) - 2 * X;
   struct Plane {
-    float v[3][3];  // [row][x - 1, x, x + 1]
+    float m[3];   // x - 1 of the three rows
+    float2 c[3];  // x, x + 1
   };
   auto load = [&](int z, Plane& p) {
     const float* q = f + wrapi(z, df.nz) * pst;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      const float2 c = __ldg(reinterpret_cast<const float2*>(q + row[k] + 2 * X));
-      p.v[k][0] = __ldg(q + row[k] + xm);
-      p.v[k][1] = c.x;
-      p.v[k][2] = c.y;
+      p.c[k] = __ldg(reinterpret_cast<const float2*>(q + row[k]));
+      p.m[k] = __ldg(q + row[k] + xm);
     }
   };
-  Plane a, b, c;
+  Plane a, b, c, nb, nc;
   load(2 * Z0 - 1, a);
+  load(2 * Z0, b);
+  load(2 * Z0 + 1, c);
   for (int Z = Z0; Z < Z1; ++Z) {
-    load(2 * Z, b);
-    load(2 * Z + 1, c);
-    float yv[3];
-#pragma unroll
-    for (int x = 0; x < 3; ++x) {
-      float zv[3];
-#pragma unroll
-      for (int k = 0; k < 3; ++k) zv[k] = fw3(a.v[k][x], b.v[k][x], c.v[k][x]);
-      yv[x] = fw3(zv[0], zv[1], zv[2]);
-    }
-    const float v = fw3(yv[0], yv[1], yv[2]);
     const long long i = lin(dc, X, Y, Z);
+    const float Jv = e1 ? __ldg(J + i) : 1.f, Dv = e1 ? __ldg(D + i) : 1.f;
+    if (Z + 1 < Z1) {
+      load(2 * Z + 2, nb);
+      load(2 * Z + 3, nc);
+    }
+    float zm[3], z0[3], zp[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      zm[k] = fw3(a.m[k], b.m[k], c.m[k]);
+      z0[k] = fw3(a.c[k].x, b.c[k].x, c.c[k].x);
+      zp[k] = fw3(a.c[k].y, b.c[k].y, c.c[k].y);
+    }
+    const float v = fw3(fw3(zm[0], zm[1], zm[2]), fw3(z0[0], z0[1], z0[2]), fw3(zp[0], zp[1], zp[2]));
     rc[i] = v;
-    if (e1) e1[i] = jacobi_value(0.f, v, J[i], D[i], 0.f, h2, omega);
+    if (e1) e1[i] = jacobi_value(0.f, v, Jv, Dv, 0.f, h2, omega);
     a = c;
+    b = nb;
+    c = nc;
   }
 }
 
@@ -1369,10 +1376,11 @@ cudaError_t launch_curv_jacobi_zero(cudaStream_t st, Dims d, const CurvCoef& cf,
 cudaError_t launch_curv_restrict(cudaStream_t st, Dims fine, const float* f, float* rc, const CurvCoef& cc, float* e1,
                                  float omega) {
   const Dims dc{fine.nx / 2, fine.ny / 2, fine.nz / 2};
-  const long long cols = (long long)((dc.nx + BX - 1) / BX) * ((dc.ny + BY - 1) / BY);
+  // the longest run of up to 8 planes that leaves six CTAs per SM
+  const long long cols = (long long)((dc.nx + BX - 1) / BX) * ((dc.ny + RBY - 1) / RBY);
   int zc = 8;
-  while (zc > 1 && cols * ((dc.nz + zc - 1) / zc) < 4 * 152) zc /= 2;
-  k_curv_restrict<<<dim3((dc.nx + BX - 1) / BX, (dc.ny + BY - 1) / BY, (dc.nz + zc - 1) / zc), dim3(BX, BY), 0, st>>>(
+  while (zc > 1 && cols * ((dc.nz + zc - 1) / zc) < 6 * 152) zc /= 2;
+  k_curv_restrict<<<dim3((dc.nx + BX - 1) / BX, (dc.ny + RBY - 1) / RBY, (dc.nz + zc - 1) / zc), dim3(BX, RBY), 0, st>>>(
       fine, f, rc, e1, cc.J, cc.D, cc.h2, omega, zc);
   note_launch();
   return cudaGetLastError();
