@@ -226,10 +226,10 @@ gbmg_status gbmg::curv_solve(gbmg_ctx* c, const double* F, double* phi, double t
 
 namespace {
 
-// The operator's diagonal on every level that is smoothed.
+// The operator's diagonal on every level (the V-cycle does not smooth the coarsest, but
+// mg_curv_smooth takes it too).
 gbmg_status build_diag(gbmg_ctx* c) {
-  for (int l = 0; l + 1 < c->L; ++l) {
-    const Level& L = c->lv[l];
+  for (const Level& L : c->lv) {
     TRY(launch_curv_diag(c->stream, L.d, L.cc, curv_form(c, false), (float*)L.cc.D));
   }
   return GBMG_OK;
