@@ -131,7 +131,9 @@ gbmg_status mg_set_stream(gbmg_ctx* ctx, void* cuda_stream);
  * orientation) and launched once per solve, and the host waits once.  While kernel families
  * are timed (mg_profile_begin), each cycle of a mixed solve is a graph launch of its own
  * with event nodes, and the host checks convergence after every cycle.  Results are the
- * same bits either way.  enable = 0 launches every kernel of every cycle from the host. */
+ * same bits either way.  enable = 0 launches every kernel of every cycle from the host;
+ * enable = 2 (testing) lets the construction of a loop fail, which leaves the context on a
+ * graph launch per cycle, as a driver that refuses it would. */
 gbmg_status mg_set_cycle_graphs(gbmg_ctx* ctx, int enable);
 
 /* Curvilinear contexts only: set the deformation potential psi (nx*ny*nz doubles,
@@ -300,7 +302,9 @@ gbmg_status mg_batch_get_tiles(const gbmg_batch* batch, int* tile_cells, int nle
  * the batch's own, replayed while tol, max_vcycles, grid and tile sizes are unchanged;
  * ordered after earlier and before later work on the batch's stream).  Where every problem
  * has a bottom cycle (degrees 1 to 4) the graph runs the phases as kernels of their own
- * in a loop on the device, otherwise the persistent kernel.  Off by default. */
+ * in a loop on the device, otherwise the persistent kernel.  on = 2 (testing) lets the
+ * construction of the phase graph fail, which leaves the batch on the persistent kernel.  Off
+ * by default. */
 gbmg_status mg_batch_use_graph(gbmg_batch* batch, int on);
 /* Number of levels of the deepest problem (length of the tile-size array). */
 int mg_batch_num_levels(const gbmg_batch* batch);

@@ -508,7 +508,7 @@ struct gbmg_batch {
   // CUDA graph of one solve (copy-in, resets, the phase kernels in a device-side loop or,
   // where they do not apply, the cooperative launch, copy-out), captured on a private stream
   // and replayed while its key is unchanged
-  bool use_graph = false;
+  bool use_graph = false, refuse = false;   // refuse (testing): building the phase graph fails
   cudaStream_t gstream = nullptr;
   cudaEvent_t gev[2] = {nullptr, nullptr};
   cudaGraphExec_t gexec = nullptr;
@@ -862,6 +862,7 @@ extern "C" gbmg_status mg_batch_set_blocks(gbmg_batch* b, int blocks) {
 extern "C" gbmg_status mg_batch_use_graph(gbmg_batch* b, int on) {
   if (!b) return fail(GBMG_ERR_INVALID_ARG, "mg_batch_use_graph: NULL batch");
   b->use_graph = on != 0;
+  b->refuse = on == 2;
   return GBMG_OK;
 }
 
@@ -933,7 +934,7 @@ extern "C" gbmg_status mg_batch_solve(gbmg_batch* b, const double* const* src_de
       // (an incomplete phase graph, say on a driver without conditional nodes, leaves the
       // batch on the persistent kernel)
       if (b->phases.usable && b->phases.build(b->gstream, D, &graph, [&]() { return copy_in(b->gstream); },
-                                              [&]() { return copy_out(b->gstream); }) != GBMG_OK) {
+                                              [&]() { return copy_out(b->gstream); }, b->refuse) != GBMG_OK) {
         if (graph) cudaGraphDestroy(graph);
         graph = nullptr;
         b->phases.usable = false;

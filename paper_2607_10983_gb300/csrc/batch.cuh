@@ -142,9 +142,9 @@ struct PhaseGraph {
   // bottom: shared memory of the largest bottom cycle
   gbmg_status init(const std::vector<gbmg_ctx*>& ctx, const BProb* prob, const BDesc& D, size_t bottom);
   // *graph: one solve, captured on gs, with head() before it and tail() after it (also set on
-  // an error, for the caller to destroy)
+  // an error, for the caller to destroy); refuse (testing): fails in the loop's capture
   gbmg_status build(cudaStream_t gs, const BDesc& D, cudaGraph_t* graph, const std::function<gbmg_status()>& head,
-                    const std::function<gbmg_status()>& tail) const;
+                    const std::function<gbmg_status()>& tail, bool refuse) const;
   ~PhaseGraph();
 };
 

@@ -16,6 +16,7 @@
 #include <algorithm>
 
 #include "batch.cuh"
+#include "loop.h"
 #include "small_cta.cuh"
 
 namespace gbmg {
@@ -351,34 +352,17 @@ gbmg_status PhaseGraph::init(const std::vector<gbmg_ctx*>& ctx, const BProb* pro
 }
 
 gbmg_status PhaseGraph::build(cudaStream_t gs, const BDesc& D, cudaGraph_t* graph,
-                              const std::function<gbmg_status()>& head, const std::function<gbmg_status()>& tail) const {
+                              const std::function<gbmg_status()>& head, const std::function<gbmg_status()>& tail,
+                              bool refuse) const {
   const Kernels K = kernels_of(D.degree);
   const int chunks = std::min(D.nchunk[0], 8 * SMS);
-  cudaGraph_t g = nullptr, ended = nullptr;
+  cudaGraph_t g = nullptr, turn = nullptr;
   TRY(cudaGraphCreate(&g, 0));
   *graph = g;
   cudaGraphConditionalHandle w;
   TRY(cudaGraphConditionalHandleCreate(&w, g, 0, cudaGraphCondAssignDefault));
-  // captures body() into `into` after `dep`; `last`: the node it ends with
-  auto record = [&](cudaGraph_t into, cudaGraphNode_t* dep, const std::function<gbmg_status()>& body,
-                    cudaGraphNode_t* last) -> gbmg_status {
-    TRY(cudaStreamBeginCaptureToGraph(gs, into, dep, nullptr, dep ? 1 : 0, cudaStreamCaptureModeThreadLocal));
-    gbmg_status s = body();
-    cudaStreamCaptureStatus cs;
-    const cudaGraphNode_t* deps = nullptr;
-    const cudaGraphEdgeData* edges = nullptr;
-    size_t nd = 0;
-    cudaError_t e = cudaStreamGetCaptureInfo(gs, &cs, nullptr, nullptr, &deps, &edges, &nd);
-    if (e == cudaSuccess && nd == 1) *last = deps[0];
-    else if (e == cudaSuccess) e = cudaErrorUnknown;
-    const cudaError_t e2 = cudaStreamEndCapture(gs, &ended);
-    if (s != GBMG_OK) return s;
-    TRY(e);
-    TRY(e2);
-    return GBMG_OK;
-  };
   cudaGraphNode_t last, loop;
-  TRYS(record(g, nullptr, [&]() -> gbmg_status {
+  TRYS(add_captured(gs, g, nullptr, [&]() -> gbmg_status {
     TRYS(head());
     k_batch_prologue<<<chunks, ET, 0, gs>>>(D);
     k_batch_mean<<<D.count, 256, 0, gs>>>(D, P_MEAN);
@@ -387,13 +371,8 @@ gbmg_status PhaseGraph::build(cudaStream_t gs, const BDesc& D, cudaGraph_t* grap
     TRY(cudaGetLastError());
     return GBMG_OK;
   }, &last));
-  cudaGraphNodeParams cp = {};
-  cp.type = cudaGraphNodeTypeConditional;
-  cp.conditional.handle = w;
-  cp.conditional.type = cudaGraphCondTypeWhile;
-  cp.conditional.size = 1;
-  TRY(cudaGraphAddNode(&loop, g, &last, nullptr, 1, &cp));
-  TRYS(record(cp.conditional.phGraph_out[0], nullptr, [&]() -> gbmg_status {
+  TRYS(add_conditional(g, last, w, cudaGraphCondTypeWhile, &turn, &loop));
+  TRYS(add_captured(gs, turn, nullptr, [&]() -> gbmg_status {
     for (int l = 0; l + 1 < D.maxL; ++l)
       if (t.dtot[l])
         K.down<<<(int)std::min<long long>(t.dtot[l], SMS), K.down_t, K.down_sm, gs>>>(D, t, l, coef[l]);
@@ -403,9 +382,10 @@ gbmg_status PhaseGraph::build(cudaStream_t gs, const BDesc& D, cudaGraph_t* grap
     k_batch_df<false><<<t.ftot, GDf::NT, kDfSmem, gs>>>(D, t);
     k_batch_books<false><<<1, 1024, 0, gs>>>(D, t, w);
     TRY(cudaGetLastError());
+    if (refuse) TRY(cudaStreamSynchronize(gs));  // (refused: the stream is captured)
     return GBMG_OK;
   }, &last));
-  TRYS(record(g, &loop, [&]() -> gbmg_status {
+  TRYS(add_captured(gs, g, &loop, [&]() -> gbmg_status {
     k_batch_phi_sum<<<chunks, ET, 0, gs>>>(D);
     k_batch_mean<<<D.count, 256, 0, gs>>>(D, P_MPHI);
     k_batch_output<<<chunks, ET, 0, gs>>>(D);
