@@ -825,7 +825,9 @@ extern "C" gbmg_status mg_batch_create(gbmg_batch** out, gbmg_ctx* const* ctxs, 
     D.small = reinterpret_cast<const SmallCycle*>(b->mem2 + oSmall);
   }
   if (b->smem > 0) {
-    e = cudaFuncSetAttribute(b->kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->smem);
+    // (the kernel's limit, which other batches share: room for the largest bottom cycle)
+    const size_t most = std::max(b->smem, kSmallSmem);
+    e = cudaFuncSetAttribute(b->kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
     if (e != cudaSuccess) {
       delete b;
       return cuda_fail(e, "mg_batch_create: shared-memory attribute");

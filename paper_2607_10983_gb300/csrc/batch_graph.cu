@@ -345,7 +345,9 @@ gbmg_status PhaseGraph::init(const std::vector<gbmg_ctx*>& ctx, const BProb* pro
   };
   TRY(smem((const void*)K.down, K.down_sm));
   TRY(smem((const void*)K.up, K.up_sm));
-  TRY(smem((const void*)k_batch_bottom, bottom_sm));
+  // (the limit belongs to the kernel, not to this batch: a smaller bottom cycle's size would
+  // refuse the launches of a batch made before)
+  TRY(smem((const void*)k_batch_bottom, kSmallSmem));
   TRY(smem((const void*)k_batch_df<true>, kDfSmem));
   TRY(smem((const void*)k_batch_df<false>, kDfSmem));
   return GBMG_OK;
