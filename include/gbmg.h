@@ -302,9 +302,9 @@ gbmg_status mg_batch_get_tiles(const gbmg_batch* batch, int* tile_cells, int nle
  * the batch's own, replayed while tol, max_vcycles, grid and tile sizes are unchanged;
  * ordered after earlier and before later work on the batch's stream).  Where every problem
  * has a bottom cycle (degrees 1 to 4) the graph runs the phases as kernels of their own
- * in a loop on the device, otherwise the persistent kernel.  on = 2 (testing) lets the
- * construction of the phase graph fail, which leaves the batch on the persistent kernel.  Off
- * by default. */
+ * in a loop on the device, otherwise the persistent kernel.  on = 2 or 3 (testing) lets the
+ * construction or the instantiation of the phase graph fail, which leaves the batch on the
+ * persistent kernel.  Off by default. */
 gbmg_status mg_batch_use_graph(gbmg_batch* batch, int on);
 /* Number of levels of the deepest problem (length of the tile-size array). */
 int mg_batch_num_levels(const gbmg_batch* batch);

@@ -508,7 +508,8 @@ struct gbmg_batch {
   // CUDA graph of one solve (copy-in, resets, the phase kernels in a device-side loop or,
   // where they do not apply, the cooperative launch, copy-out), captured on a private stream
   // and replayed while its key is unchanged
-  bool use_graph = false, refuse = false;   // refuse (testing): building the phase graph fails
+  bool use_graph = false;
+  int refuse = 0;   // testing: building (2) or instantiating (3) the phase graph fails
   cudaStream_t gstream = nullptr;
   cudaEvent_t gev[2] = {nullptr, nullptr};
   cudaGraphExec_t gexec = nullptr;
@@ -864,7 +865,7 @@ extern "C" gbmg_status mg_batch_set_blocks(gbmg_batch* b, int blocks) {
 extern "C" gbmg_status mg_batch_use_graph(gbmg_batch* b, int on) {
   if (!b) return fail(GBMG_ERR_INVALID_ARG, "mg_batch_use_graph: NULL batch");
   b->use_graph = on != 0;
-  b->refuse = on == 2;
+  b->refuse = on;
   return GBMG_OK;
 }
 
@@ -933,17 +934,23 @@ extern "C" gbmg_status mg_batch_solve(gbmg_batch* b, const double* const* src_de
         b->gexec = nullptr;
       }
       cudaGraph_t graph = nullptr;
-      // (an incomplete phase graph, say on a driver without conditional nodes, leaves the
-      // batch on the persistent kernel)
-      if (b->phases.usable && b->phases.build(b->gstream, D, &graph, [&]() { return copy_in(b->gstream); },
-                                              [&]() { return copy_out(b->gstream); }, b->refuse) != GBMG_OK) {
+      // (a phase graph that cannot be built or instantiated, say on a driver without conditional
+      // nodes or with no memory left for them, leaves the batch on the persistent kernel)
+      if (b->phases.usable) {
+        gbmg_status ps = b->phases.build(b->gstream, D, &graph, [&]() { return copy_in(b->gstream); },
+                                         [&]() { return copy_out(b->gstream); }, b->refuse == 2);
+        if (ps == GBMG_OK && (b->refuse == 3 || cudaGraphInstantiate(&b->gexec, graph, 0) != cudaSuccess))
+          ps = GBMG_ERR_CUDA;
         if (graph) cudaGraphDestroy(graph);
         graph = nullptr;
-        b->phases.usable = false;
-        (void)cudaGetLastError();
-        g_last_error.clear();
+        if (ps != GBMG_OK) {
+          b->gexec = nullptr;
+          b->phases.usable = false;
+          (void)cudaGetLastError();
+          g_last_error.clear();
+        }
       }
-      if (!b->phases.usable) {
+      if (!b->gexec) {
         TRY(cudaStreamBeginCapture(b->gstream, cudaStreamCaptureModeThreadLocal));
         const gbmg_status cs = enqueue(b->gstream);
         const cudaError_t ce = cudaStreamEndCapture(b->gstream, &graph);
@@ -952,10 +959,11 @@ extern "C" gbmg_status mg_batch_solve(gbmg_batch* b, const double* const* src_de
           return cs;
         }
         TRY(ce);
+        const cudaError_t ie = cudaGraphInstantiate(&b->gexec, graph, 0);
+        cudaGraphDestroy(graph);
+        if (ie != cudaSuccess) b->gexec = nullptr;
+        TRY(ie);
       }
-      const cudaError_t ie = cudaGraphInstantiate(&b->gexec, graph, 0);
-      cudaGraphDestroy(graph);
-      TRY(ie);
       b->g_version = b->version;
       b->g_tol = tol;
       b->g_maxv = D.maxv;

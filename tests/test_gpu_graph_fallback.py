@@ -46,13 +46,14 @@ def test_curvilinear_solve_without_its_loop(gb, sym):
         assert all(torch.equal(a, b) for a, b in zip(got[0][:3], got[1][:3]))
 
 
+@pytest.mark.parametrize("refusal", [2, 3])   # of its construction, of its instantiation
 @pytest.mark.parametrize("degree", [1, 3])
-def test_batch_without_its_phase_graph(gb, degree):
+def test_batch_without_its_phase_graph(gb, degree, refusal):
     shapes = [(32, 32, 32), (64, 48, 64)]
     F = [torch.from_numpy(grf(s, 324 + i)).cuda() for i, s in enumerate(shapes)]
     batch = gb.Batch(shapes, degree=degree)
     got = []
-    for mode in (0, 2, 2):
+    for mode in (0, refusal, refusal):
         gb._check(gb.lib().mg_batch_use_graph(batch._b, mode))
         phi = [torch.zeros_like(f) for f in F]
         stats, _ = batch.solve(F, phi, tol=1e-8)
