@@ -299,10 +299,11 @@ gbmg_status mg_batch_set_tiles(gbmg_batch* batch, const int* tile_cells, int nle
 /* Current tile sizes of levels 0 .. nlevels-1 (0 beyond the deepest level). */
 gbmg_status mg_batch_get_tiles(const gbmg_batch* batch, int* tile_cells, int nlevels);
 /* on != 0: run each solve as a CUDA graph (captured at the first solve on a stream of
- * the batch's own, replayed while tol, max_vcycles, grid and tile sizes are unchanged;
- * ordered after earlier and before later work on the batch's stream).  Where every problem
- * has a bottom cycle (degrees 1 to 4) the graph runs the phases as kernels of their own
- * in a loop on the device, otherwise the persistent kernel.  on = 2 or 3 (testing) lets the
+ * the batch's own, replayed while tol, max_vcycles and what it reads of the grid and tile
+ * sizes are unchanged; ordered after earlier and before later work on the batch's stream).
+ * Where every problem has even nx, a bottom cycle (degrees 1 to 4) and no level above it with
+ * a side below 16, the graph runs the phases as kernels of their own in a loop on the device
+ * (of the grid and tile sizes it reads the level-0 tiles), otherwise the persistent kernel.  on = 2 or 3 (testing) lets the
  * construction or the instantiation of the phase graph fail, which leaves the batch on the
  * persistent kernel.  Off by default. */
 gbmg_status mg_batch_use_graph(gbmg_batch* batch, int on);
@@ -312,7 +313,8 @@ int mg_batch_num_levels(const gbmg_batch* batch);
  * (1 .. resident blocks per SM, times the SM count), then, level by level, the tile
  * size (1024, 2048, ... 65536 cells).  Every trial starts from the initial guesses in
  * phi_dev (saved in temporary device buffers, released before returning); on return
- * phi_dev holds the solution from those guesses with the chosen settings.
+ * phi_dev holds the solution from those guesses with the chosen settings.  Settings that the
+ * batch's graph does not read (mg_batch_use_graph) stay as they are.
  * *blocks_out and tiles_out[0 .. levels-1] (both nullable) receive the choice. */
 gbmg_status mg_batch_autotune(gbmg_batch* batch, const double* const* source_dev, double* const* phi_dev,
                               double tol, int max_vcycles, int* blocks_out, int* tiles_out);

@@ -507,7 +507,9 @@ struct gbmg_batch {
   size_t res_bytes = 0;
   // CUDA graph of one solve (copy-in, resets, the phase kernels in a device-side loop or,
   // where they do not apply, the cooperative launch, copy-out), captured on a private stream
-  // and replayed while its key is unchanged
+  // and replayed while its key is unchanged: the tolerance, the cycle limit and what its form
+  // reads of the schedule (the phases: the level-0 tile size; the persistent kernel: the grid
+  // and every tile size)
   bool use_graph = false;
   int refuse = 0;   // testing: building (2) or instantiating (3) the phase graph fails
   cudaStream_t gstream = nullptr;
@@ -515,7 +517,8 @@ struct gbmg_batch {
   cudaGraphExec_t gexec = nullptr;
   unsigned version = 0, g_version = ~0u;
   double g_tol = -1.0;
-  int g_maxv = -1, g_blocks = -1;
+  int g_maxv = -1, g_blocks = -1, g_chunk0 = 0;
+  bool g_phases = false;   // the captured graph is the phase graph
   // kernel for the batch's degree and its dynamic shared memory; device memory of the
   // second phi buffers and the fused-phase tables
   const void* kern = nullptr;
@@ -927,8 +930,9 @@ extern "C" gbmg_status mg_batch_solve(gbmg_batch* b, const double* const* src_de
       TRY(cudaEventCreateWithFlags(&b->gev[0], cudaEventDisableTiming));
       TRY(cudaEventCreateWithFlags(&b->gev[1], cudaEventDisableTiming));
     }
-    if (!b->gexec || b->g_version != b->version || b->g_tol != tol || b->g_maxv != D.maxv ||
-        b->g_blocks != b->blocks) {
+    const bool current = b->g_phases ? b->g_chunk0 == D.chunk[0]
+                                     : b->g_version == b->version && b->g_blocks == b->blocks;
+    if (!b->gexec || !current || b->g_tol != tol || b->g_maxv != D.maxv) {
       if (b->gexec) {
         cudaGraphExecDestroy(b->gexec);
         b->gexec = nullptr;
@@ -950,6 +954,8 @@ extern "C" gbmg_status mg_batch_solve(gbmg_batch* b, const double* const* src_de
           g_last_error.clear();
         }
       }
+      b->g_phases = b->gexec != nullptr;
+      b->g_chunk0 = D.chunk[0];
       if (!b->gexec) {
         TRY(cudaStreamBeginCapture(b->gstream, cudaStreamCaptureModeThreadLocal));
         const gbmg_status cs = enqueue(b->gstream);
@@ -1000,15 +1006,17 @@ extern "C" gbmg_status mg_batch_solve(gbmg_batch* b, const double* const* src_de
 
 namespace {
 
-// One timed trial from the saved initial guesses.
+// One timed trial from the saved initial guesses (with graphs, a first solve captures it untimed).
 gbmg_status trial(gbmg_batch* b, const double* const* src, double* const* phi, double* const* save, double tol,
                   int maxv, cudaEvent_t e0, cudaEvent_t e1, float& ms) {
-  for (int i = 0; i < b->count; ++i)
-    TRY(cudaMemcpyAsync(phi[i], save[i], sizeof(double) * ncell(b->ctx[i]->lv[0].d), cudaMemcpyDeviceToDevice,
-                        b->stream));
-  TRY(cudaEventRecord(e0, b->stream));
-  const gbmg_status s = mg_batch_solve(b, src, phi, tol, maxv, nullptr, nullptr);
-  if (s == GBMG_ERR_CUDA || s == GBMG_ERR_INVALID_ARG || s == GBMG_ERR_OOM) return s;
+  for (int pass = b->use_graph ? 0 : 1; pass < 2; ++pass) {
+    for (int i = 0; i < b->count; ++i)
+      TRY(cudaMemcpyAsync(phi[i], save[i], sizeof(double) * ncell(b->ctx[i]->lv[0].d), cudaMemcpyDeviceToDevice,
+                          b->stream));
+    TRY(cudaEventRecord(e0, b->stream));
+    const gbmg_status s = mg_batch_solve(b, src, phi, tol, maxv, nullptr, nullptr);
+    if (s == GBMG_ERR_CUDA || s == GBMG_ERR_INVALID_ARG || s == GBMG_ERR_OOM) return s;
+  }
   TRY(cudaEventRecord(e1, b->stream));
   TRY(cudaEventSynchronize(e1));
   TRY(cudaEventElapsedTime(&ms, e0, e1));
@@ -1037,16 +1045,21 @@ extern "C" gbmg_status mg_batch_autotune(gbmg_batch* b, const double* const* src
     TRY(cudaEventCreate(&e0));
     TRY(cudaEventCreate(&e1));
     float ms = 0.f, best_ms = -1.f;
+    // (with graphs, a first trial shows whether the phase graph serves: of the schedule it reads
+    // the level-0 tile size alone, and trials of the rest would compare equal solves)
+    if (b->use_graph) TRYS(trial(b, src_dev, phi_dev, save.data(), tol, max_vcycles, e0, e1, ms));
+    const bool phases = b->use_graph && b->gexec && b->g_phases;
+    if (phases) best_ms = ms;
     // grid size: 1 .. (resident blocks per SM) times the SM count
     int best = b->blocks;
-    for (int blocks = sms; blocks <= most; blocks += sms) {
+    for (int blocks = sms; blocks <= most && !phases; blocks += sms) {
       b->blocks = blocks;
       TRYS(trial(b, src_dev, phi_dev, save.data(), tol, max_vcycles, e0, e1, ms));
       if (best_ms < 0.f || ms < best_ms) best_ms = ms, best = blocks;
     }
     b->blocks = best;
     // tile size per level, one level at a time (coordinate descent from the current sizes)
-    for (int l = 0; l < b->maxL; ++l) {
+    for (int l = 0; l < (phases ? 1 : b->maxL); ++l) {
       long long biggest = 0;
       for (auto* c : b->ctx)
         if (l < c->L) biggest = std::max(biggest, ncell(c->lv[l].d));
