@@ -28,6 +28,7 @@ namespace {
 constexpr int NB = 8;        // columns of a panel
 constexpr int PT = 32 * NB;  // threads of a CTA
 constexpr int kMaxPolls = 1 << 20;
+constexpr int kMaxN = 512;   // unknowns of a coarsest level at most (mg_setup)
 
 // Zero and NaN by the bits: FP64 comparisons run in the slow FP64 pipe, whose occupancy is
 // what the elimination waits for.
@@ -252,7 +253,8 @@ cudaError_t launch_coarse_inverse(cudaStream_t st, int n, const double* dense, v
   double* F = X + 2 * (size_t)m * m;
   Step* S = (Step*)(F + 2 * cols * m);
   int* flag = (int*)(S + 2 * cols);
-  cudaError_t e = cudaFuncSetAttribute(k_invert, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  // (the limit belongs to the kernel: the largest size, whatever other threads invert)
+  cudaError_t e = cudaFuncSetAttribute(k_invert, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes(kMaxN));
   if (e == cudaSuccess) e = cudaMemsetAsync(status, 0, sizeof(int), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(flag, 0, 2 * panels * sizeof(int), st);
   if (e != cudaSuccess) return e;
