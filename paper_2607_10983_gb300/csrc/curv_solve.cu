@@ -11,6 +11,7 @@
 // delta_bar = J (lam - sum(J lam)/sum(J)), psi_bar through the geometry.
 // With the symmetric variant (opts.curv_sym) both solves use S, its own transpose.
 #include <cstring>
+#include <vector>
 
 #include "kernels.h"
 #include "loop.h"
@@ -235,6 +236,27 @@ gbmg_status build_diag(gbmg_ctx* c) {
   return GBMG_OK;
 }
 
+// The coarsest inverses on the host, where the GPU has no room for the kernel's resident grid
+// (up to 130 CTAs: a partition of a few SMs).  The same bits.
+gbmg_status coarsest_on_host(gbmg_ctx* c, const char* who) {
+  const size_t nc = c->nc, n2 = nc * nc;
+  std::vector<float> Jc(nc);
+  std::vector<double> Lm(n2), G;
+  TRY(cudaMemcpyAsync(Jc.data(), c->lv[c->L - 1].cc.J, nc * sizeof(float), cudaMemcpyDeviceToHost, c->stream));
+  for (int tr = 0; tr < 2; ++tr) {
+    TRY(cudaMemcpyAsync(Lm.data(), c->dense + tr * n2, n2 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+    TRY(cudaStreamSynchronize(c->stream));
+    for (float v : Jc)
+      if (!(v > 0.f)) return fail(GBMG_ERR_INVALID_ARG, std::string(who) + ": non-positive volume element on the coarsest level");
+    const std::vector<double> w(Jc.begin(), Jc.end());
+    if (!dense_pinv((int)nc, Lm, w, G)) return fail(GBMG_ERR_INVALID_ARG, std::string(who) + ": coarsest operator is singular");
+    const std::vector<float> G32(G.begin(), G.end());
+    TRY(cudaMemcpy(tr ? c->G64T : c->G64, G.data(), n2 * sizeof(double), cudaMemcpyHostToDevice));
+    TRY(cudaMemcpy(tr ? c->G32T : c->G32, G32.data(), n2 * sizeof(float), cudaMemcpyHostToDevice));
+  }
+  return GBMG_OK;
+}
+
 // Exact inverses of the coarsest operator and of its transposed-solve twin (minimum-norm,
 // left null vector J), built from the coarsest level's coefficients.  Waits for the stream.
 gbmg_status build_coarsest(gbmg_ctx* c, const char* who) {
@@ -244,8 +266,14 @@ gbmg_status build_coarsest(gbmg_ctx* c, const char* who) {
   int* const status = reinterpret_cast<int*>(c->scal + S_PINV);
   for (int tr = 0; tr < 2; ++tr)
     TRY(launch_curv_dense(c->stream, C.d, C.cc, curv_form(c, tr != 0), c->dense + tr * n2));
-  TRY(launch_coarse_inverse(c->stream, nc, c->dense, c->dense + 2 * n2, C.cc.J, c->G64, c->G64T, c->G32, c->G32T,
-                            status));
+  const cudaError_t e = c->refuse ? cudaErrorCooperativeLaunchTooLarge
+                                  : launch_coarse_inverse(c->stream, nc, c->dense, c->dense + 2 * n2, C.cc.J, c->G64,
+                                                          c->G64T, c->G32, c->G32T, status);
+  if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+    (void)cudaGetLastError();
+    return coarsest_on_host(c, who);
+  }
+  if (e != cudaSuccess) return cuda_fail(e, "launch_coarse_inverse");
   TRY(launch_scalars_to_host(c->stream, c->scal + S_PINV, c->host_scal_dev + S_PINV, 1));
   TRY(cudaStreamSynchronize(c->stream));
   int flags;

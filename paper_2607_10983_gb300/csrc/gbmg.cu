@@ -298,7 +298,7 @@ extern "C" gbmg_status mg_set_cycle_graphs(gbmg_ctx* ctx, int enable) {
   if (e != cudaSuccess) return cuda_fail(e, "mg_set_cycle_graphs");
   ctx->cyc_off = enable == 0;
   if (enable) ctx->loop_off = false;
-  ctx->refuse_loop = enable == 2;
+  ctx->refuse = enable == 2;
   ctx->graph_mask = -1;  // drop the graphs captured so far
   sync_graph_mask(ctx);
   return GBMG_OK;

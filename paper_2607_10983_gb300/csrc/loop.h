@@ -75,7 +75,7 @@ void build_loop(gbmg_ctx* c, Cycle cycle, long long npart, cudaGraphExec_t& exec
     TRY(cudaGraphConditionalHandleCreate(&f, b0, 0, cudaGraphCondAssignDefault));
     auto body = [&](int second) -> gbmg_status {
       TRYS(cycle());
-      if (second && c->refuse_loop) TRY(cudaStreamSynchronize(c->stream));  // (refused: the stream is captured)
+      if (second && c->refuse) TRY(cudaStreamSynchronize(c->stream));  // (refused: the stream is captured)
       TRY(launch_loop_check(c->stream, c->partials, npart, c->scal + S_R2, c->loop_dev, c->loop_host_dev, w, f, second));
       return GBMG_OK;
     };
