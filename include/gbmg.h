@@ -133,7 +133,7 @@ gbmg_status mg_set_stream(gbmg_ctx* ctx, void* cuda_stream);
  * with event nodes, and the host checks convergence after every cycle.  Results are the
  * same bits either way.  enable = 0 launches every kernel of every cycle from the host;
  * enable = 2 (testing) refuses the context what a driver or a partition of a GPU may refuse:
- * loops in graphs (leaving a graph launch per cycle) and cooperative grids. */
+ * loops in graphs (leaving a graph launch per cycle), cooperative grids and clusters of 16. */
 gbmg_status mg_set_cycle_graphs(gbmg_ctx* ctx, int enable);
 
 /* Curvilinear contexts only: set the deformation potential psi (nx*ny*nz doubles,

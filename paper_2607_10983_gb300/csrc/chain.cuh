@@ -214,25 +214,41 @@ size_t layout(Fields<T>& F) {
   return off;
 }
 
-// Launch of a kernel whose CTAs form one cluster of kCtas.
+// Configuration of a kernel whose CTAs form one cluster of kCtas; its limits are set.
+struct Config {
+  cudaLaunchConfig_t c = {};
+  cudaLaunchAttribute at = {};
+};
+template <typename K>
+cudaError_t configure(Config& q, cudaStream_t st, K kernel, int threads, size_t smem) {
+  cudaError_t e = cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  q.c.gridDim = dim3(kCtas);
+  q.c.blockDim = dim3(threads);
+  q.c.dynamicSmemBytes = smem;
+  q.c.stream = st;
+  q.at.id = cudaLaunchAttributeClusterDimension;
+  q.at.val.clusterDim.x = kCtas;
+  q.at.val.clusterDim.y = q.at.val.clusterDim.z = 1;
+  q.c.attrs = &q.at;
+  q.c.numAttrs = 1;
+  return e;
+}
+// 16 CTAs are more than the portable cluster size: a device or a partition may have no room
+// for them.
+template <typename K>
+bool fits(K kernel, int threads, size_t smem) {
+  Config q;
+  int n = 0;
+  const bool ok = configure(q, nullptr, kernel, threads, smem) == cudaSuccess &&
+                  cudaOccupancyMaxActiveClusters(&n, kernel, &q.c) == cudaSuccess && n > 0;
+  if (!ok) (void)cudaGetLastError();
+  return ok;
+}
 template <typename K, typename A>
 cudaError_t launch(cudaStream_t st, K kernel, int threads, size_t smem, const A& args) {
-  cudaError_t e = cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (e == cudaSuccess && smem > 48 * 1024)
-    e = cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t c = {};
-  c.gridDim = dim3(kCtas);
-  c.blockDim = dim3(threads);
-  c.dynamicSmemBytes = smem;
-  c.stream = st;
-  cudaLaunchAttribute at;
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = kCtas;
-  at.val.clusterDim.y = at.val.clusterDim.z = 1;
-  c.attrs = &at;
-  c.numAttrs = 1;
-  e = cudaLaunchKernelEx(&c, kernel, args);
+  Config q;
+  cudaError_t e = configure(q, st, kernel, threads, smem);
+  if (e == cudaSuccess) e = cudaLaunchKernelEx(&q.c, kernel, args);
   if (e == cudaSuccess) note_launch();
   return e;
 }

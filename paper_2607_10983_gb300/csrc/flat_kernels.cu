@@ -545,8 +545,11 @@ cudaError_t launch_residual_restrict(cudaStream_t st, Dims fine, const T* f, con
   note_launch();
   return cudaGetLastError();
 }
+constexpr size_t kChainSmem = 16 * 1024;   // more than 4096 cells and the levels below them take
+bool chain_f64_fits() { return chain::fits(k_chain_f64, kChainThreads, kChainSmem); }
 cudaError_t launch_chain_f64(cudaStream_t st, chain::Fields<double> f, const ChainCheb& k) {
   const size_t smem = chain::layout(f);
+  if (smem > kChainSmem) return cudaErrorInvalidValue;
   return chain::launch(st, k_chain_f64, kChainThreads, smem, ChainArgs64{f, k});
 }
 template <typename T>

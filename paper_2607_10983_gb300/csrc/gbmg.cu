@@ -154,6 +154,7 @@ extern "C" gbmg_status mg_setup(gbmg_ctx** out, int nx, int ny, int nz, int leve
   c->L = (int)dims.size();
   c->nc = (int)nc;
   c->fused_all = o.fused == 2;
+  c->chain_ok = o.prec == GBMG_FP64 && chain_f64_fits();
   chebyshev_schedule(o.degree, o.alpha, c->cc1, c->cc2);
 
   const size_t esz = o.prec == GBMG_FP64 ? sizeof(double) : sizeof(float);

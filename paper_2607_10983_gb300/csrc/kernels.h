@@ -36,6 +36,7 @@ struct Fields;
 struct ChainCheb {   // FP64: constants per level and step
   double a[8][8], b[8][8], c1[8], ih2[8];
 };
+bool chain_f64_fits();   // the current device has room for it
 cudaError_t launch_chain_f64(cudaStream_t st, chain::Fields<double> f, const ChainCheb& k);
 // Folded Chebyshev constants of step k on a level of spacing h.
 inline void cheb_constants(double c2, double h, double& a, double& b) {

@@ -93,11 +93,11 @@ gbmg_status store_coarse_correction(gbmg_ctx* c, int l, float* e) {
 }
 
 // FP64 Chebyshev levels of at most this many cells, with at least one smoothed level, run in
-// one launch from the first step on.
+// one launch from the first step on, where the device has room for its cluster.
 constexpr long long kChainCells64 = 4096;
 bool chain64_from(const gbmg_ctx* c, int l) {
-  return c->o.smoother == GBMG_SMOOTH_CHEBYSHEV && c->o.degree >= 1 && c->o.degree <= 8 && l >= 1 && c->L - l >= 2 &&
-         c->L - l <= chain::kMaxL && ncell(c->lv[l].d) <= kChainCells64;
+  return c->chain_ok && !c->refuse && c->o.smoother == GBMG_SMOOTH_CHEBYSHEV && c->o.degree >= 1 &&
+         c->o.degree <= 8 && l >= 1 && c->L - l >= 2 && c->L - l <= chain::kMaxL && ncell(c->lv[l].d) <= kChainCells64;
 }
 gbmg_status chain64(gbmg_ctx* c, int l0, double*& e) {
   chain::Fields<double> F{};

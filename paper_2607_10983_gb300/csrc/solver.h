@@ -114,6 +114,7 @@ struct gbmg_ctx {
   cudaGraphExec_t loop_exec[2] = {nullptr, nullptr};
   long long loop_kernels[2] = {0, 0};
   bool loop_off = false;  // building a loop failed: a graph launch per cycle instead
+  bool chain_ok = false;  // FP64: the device takes the bottom's cluster launch
   bool refuse = false;    // testing: loops, cooperative grids and large clusters are refused
   gbmg::LoopState* loop_dev = nullptr;
   gbmg::LoopState* loop_host = nullptr;      // mapped host copy of the books
