@@ -514,13 +514,9 @@ template <int MODE, class OP, int R, int MINB, int UN>
 cudaError_t launch(cudaStream_t st, Dims d, const CurvCoef& cf, const float* r, const float* e, float* out,
                    float omega) {
   constexpr size_t sm = 3 * (size_t)SLOT * sizeof(float);
-  static bool attr = false;
-  if (!attr) {
-    const cudaError_t err =
-        cudaFuncSetAttribute(k_curv_march<MODE, OP, R, MINB, UN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (err != cudaSuccess) return err;
-    attr = true;
-  }
+  static DeviceSet done{0};
+  const cudaError_t err = allow_smem(done, k_curv_march<MODE, OP, R, MINB, UN>, sm);
+  if (err != cudaSuccess) return err;
   Fields P;
   P.p[FU] = e;
   for (int k = 0; k < 6; ++k) P.p[FXX + k] = cf.B[k];

@@ -490,13 +490,9 @@ __global__ void __launch_bounds__(NT, MINB) k_curv_df_march(Dims d, Fields P, Df
 constexpr int kCtas[3] = {2, 1, 2};
 template <class OP, int MINB>
 cudaError_t launch(cudaStream_t st, Dims d, const Fields& P, DfArgs A) {
-  static bool attr = false;
-  if (!attr) {
-    const cudaError_t err =
-        cudaFuncSetAttribute(k_curv_df_march<OP, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
-    if (err != cudaSuccess) return err;
-    attr = true;
-  }
+  static DeviceSet done{0};
+  const cudaError_t err = allow_smem(done, k_curv_df_march<OP, MINB>, kSmem);
+  if (err != cudaSuccess) return err;
   A.zc = march_zchunk(d, MINB * 152);
   k_curv_df_march<OP, MINB><<<march_grid(d, A.zc), NT, kSmem, st>>>(d, P, A);
   note_launch();

@@ -90,13 +90,10 @@ cudaError_t launch_df_update_residual(cudaStream_t st, Dims d, const float2* phi
                                       const double* m_dev, float2* phi_out, float* r_out, double* pr2, double* psum,
                                       double* pf2) {
   if (d.nx % 2) return cudaErrorInvalidValue;  // x-pairs
-  static bool attr = false;
   const size_t sm = 3 * (size_t)DFT::PLANE * sizeof(float);
-  if (!attr) {
-    cudaError_t err = cudaFuncSetAttribute(k_df_update_residual<DFT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (err != cudaSuccess) return err;
-    attr = true;
-  }
+  static DeviceSet done{0};
+  const cudaError_t err = allow_smem(done, k_df_update_residual<DFT>, sm);
+  if (err != cudaSuccess) return err;
   const int zc = df_zchunk(d);
   const dim3 grid((d.nx + DFT::TX - 1) / DFT::TX, (d.ny + DFT::TY - 1) / DFT::TY, (d.nz + zc - 1) / zc);
   k_df_update_residual<DFT><<<grid, DFT::NT, sm, st>>>(d, phi_in, e, F, m_dev, phi_out, r_out, pr2, psum, pf2, zc);

@@ -4,8 +4,21 @@
 #include <cuda_runtime.h>
 
 #include "common.cuh"
+#include "once.h"
 
 namespace gbmg {
+
+// Raises a kernel's limit of dynamic shared memory, once on each device; `done` belongs to the
+// kernel.
+template <class Kernel>
+cudaError_t allow_smem(DeviceSet& done, Kernel* kernel, size_t bytes) {
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  return once_per_device(done, dev, [&]() {
+    return cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  });
+}
 
 // Counts kernel launches made by this library (process-wide, for measurement).
 void note_launch();

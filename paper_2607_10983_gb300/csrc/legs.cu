@@ -79,12 +79,12 @@ k_up_fused(Dims d, const float* __restrict__ e_in, const float* __restrict__ ec,
 // ------------------------------------------------------------------ launch
 
 int sm_count() {
-  static int n = 0;
-  if (n == 0) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1)
-      n = 152;
-  }
+  static const int n = []() {
+    int dev = 0, v = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v < 1)
+      v = 152;
+    return v;
+  }();
   return n;
 }
 
@@ -108,13 +108,10 @@ Sched make_sched(Dims d, int warm, int& ctas) {
 template <int V>
 cudaError_t down_v(cudaStream_t st, Dims d, const float* r, float* e, float* rc, float ih2, const Coef& cf) {
   using TL = typename DownTile<V>::T;
-  static bool attr = false;
   const size_t sm = down_smem<V>();
-  if (!attr) {
-    cudaError_t err = cudaFuncSetAttribute(k_down_fused<V, TL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (err != cudaSuccess) return err;
-    attr = true;
-  }
+  static DeviceSet done{0};
+  const cudaError_t err = allow_smem(done, k_down_fused<V, TL>, sm);
+  if (err != cudaSuccess) return err;
   int ctas = 0;
   const Sched sc = make_sched<TL>(d, 2 * V + 3, ctas);
   k_down_fused<V, TL><<<ctas, TL::NT, sm, st>>>(d, r, e, rc, sc, ih2, cf);
@@ -126,13 +123,10 @@ template <int V>
 cudaError_t up_v(cudaStream_t st, Dims d, const float* e_in, const float* ec, const float* r, float* e_out,
                  float ih2, const Coef& cf) {
   using TL = typename UpTile<V>::T;
-  static bool attr = false;
   const size_t sm = up_smem<V>();
-  if (!attr) {
-    cudaError_t err = cudaFuncSetAttribute(k_up_fused<V, TL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (err != cudaSuccess) return err;
-    attr = true;
-  }
+  static DeviceSet done{0};
+  const cudaError_t err = allow_smem(done, k_up_fused<V, TL>, sm);
+  if (err != cudaSuccess) return err;
   int ctas = 0;
   const Sched sc = make_sched<TL>(d, 2 * V, ctas);
   k_up_fused<V, TL><<<ctas, TL::NT, sm, st>>>(d, e_in, ec, r, e_out, sc, ih2, cf);

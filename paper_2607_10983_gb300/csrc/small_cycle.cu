@@ -26,12 +26,9 @@ cudaError_t launch_small_vcycle(cudaStream_t st, const SmallCycle& P, const floa
     return cudaErrorInvalidValue;
   const size_t sm = small_cycle_smem(P);
   if (sm > kSmallSmem) return cudaErrorInvalidValue;
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t err = cudaFuncSetAttribute(k_small_vcycle, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallSmem);
-    if (err != cudaSuccess) return err;
-    attr = true;
-  }
+  static DeviceSet done{0};
+  const cudaError_t err = allow_smem(done, k_small_vcycle, kSmallSmem);
+  if (err != cudaSuccess) return err;
   k_small_vcycle<<<1, kSmallThreads, sm, st>>>(P, r_in, e_out);
   note_launch();
   return cudaGetLastError();
