@@ -58,10 +58,8 @@ __device__ double gradT_f64(const float* w, Dims d, int x, int y, int z, int ord
 // against 0.05 ms of memory traffic.  So the numerator N = 12 grad^T w (order 2: 2
 // grad^T w), a sum of FP32 values with power-of-two weights, is accumulated as an
 // expansion of three FP32 parts on packed x-pairs (exact to 2^-72, beyond FP64), and
-// turned into the FP64 quotient by integer operations.  The dot product is summed by
-// parts, sum(w . grad u) = sum(u grad^T w): one FP64 multiply-add per cell.  At 256^3:
-// transpose 0.156 ms, dot product 0.258 ms, both bound by instruction issue (about 190
-// FP32 additions and 60 integer operations per pair of cells).
+// turned into the FP64 quotient by integer operations.  At 256^3: 0.156 ms, bound by
+// instruction issue (about 190 FP32 additions and 60 integer operations per pair of cells).
 
 // Sum of three FP32 parts s + c + c2, |c2| << |c| << |s|, lane by lane.
 struct PAcc3 {
@@ -213,7 +211,23 @@ __global__ void k_grad_T(Dims d, const float* __restrict__ w, double* __restrict
   });
 }
 
-// block partials of sum(u grad^T w) = sum(w . grad u)
+// (double)f by integer operations (conversions run at the FP64 pipe's rate), f zero or normal.
+__device__ __forceinline__ bool widens(float f) {
+  const unsigned m = __float_as_uint(f) & 0x7fffffffu;
+  return m == 0u || (m >= 0x00800000u && m < 0x7f800000u);
+}
+__device__ __forceinline__ double widen(float f) {
+  const unsigned b = __float_as_uint(f), m = b & 0x7fffffffu;
+  return __hiloint2double((int)((m ? (m >> 3) + 0x38000000u : 0u) | (b & 0x80000000u)), (int)(b << 29));
+}
+
+// Block partials of sum(w . grad u), from differences of u.  The sum of u grad^T w over the cells
+// is the same number, but its terms have u's size instead of its gradient's: 15 times the
+// error on a potential of 160^3 (spectrum k^-6), 10 times with a constant in u.  Here a constant
+// drops out of the differences before anything else.  12 FP64 operations per cell (order 4; the
+// divisions wait for the block's sum) bound it at the FP64 pipe's 1.6 per clock and SM: 0.407 ms
+// at 256^3, order 2 0.208 (0.51 and 0.31 with the conversions of w in that pipe; one cell per
+// thread with its divisions and a block reduction 1.36; the sum of u grad^T w 0.27 and 0.16).
 template <int ORDER, int W>
 __global__ void k_grad_dot(Dims d, const double* __restrict__ u, const float* __restrict__ w,
                            double* __restrict__ partials, int gz) {
@@ -222,20 +236,70 @@ __global__ void k_grad_dot(Dims d, const double* __restrict__ u, const float* __
   double v = 0.0;
   if (x < d.nx && y < d.ny) {
     const int z0 = blockIdx.z * gz, zend = min(z0 + gz, d.nz);
-    const double* const up = u + (long long)y * d.nx + x;
-    const long long pst = (long long)d.nx * d.ny;
-    gradT_column<ORDER, W>(d, w, x, y, z0, zend, [&](int z, double v0, double v1) {
-      if constexpr (W == 2) {
-        const double2 q = *reinterpret_cast<const double2*>(up + z * pst);
-        v = fma(q.x, v0, v);
-        v = fma(q.y, v1, v);
-      } else {
-        v = fma(up[z * pst], v0, v);
+    const long long n = ncell(d), pst = (long long)d.nx * d.ny;
+    auto ldu = [&](const double* p) -> double2 {
+      if constexpr (W == 2) return __ldg(reinterpret_cast<const double2*>(p));
+      else return make_double2(__ldg(p), 0.0);
+    };
+    auto ldw = [&](const float* p) -> float2 {
+      if constexpr (W == 2) return __ldg(reinterpret_cast<const float2*>(p));
+      else return make_float2(__ldg(p), 0.f);
+    };
+    // w times the stencil's numerator; both differences first: a constant in u drops out
+    auto term = [](double& s, double wv, double m2, double m1, double p1, double p2) {
+      const double q = ORDER == 4 ? fma(8.0, p1 - m1, -(p2 - m2)) : p1 - m1;
+      s = fma(wv, q, s);
+    };
+    double vx = 0.0, vy = 0.0, vz = 0.0;
+    const long long row = (long long)y * d.nx, i = row + x;
+    // the x neighbours: of the pair, its two neighbouring pairs
+    const long long xm = row + wrap2(x - (W == 2 ? 2 : 1), d.nx), xp = row + wrap2(x + (W == 2 ? 2 : 1), d.nx);
+    const long long xmm = row + wrap2(x - 2, d.nx), xpp = row + wrap2(x + 2, d.nx);  // W = 1
+    const long long ym = (long long)wrap2(y - 1, d.ny) * d.nx + x, yp = (long long)wrap2(y + 1, d.ny) * d.nx + x;
+    const long long ymm = (long long)wrap2(y - 2, d.ny) * d.nx + x, ypp = (long long)wrap2(y + 2, d.ny) * d.nx + x;
+    double2 c[5];  // u at planes z - 2 .. z + 2
+#pragma unroll
+    for (int k = 0; k < 4; ++k) c[k + 1] = ldu(u + wrap2(z0 - 2 + k, d.nz) * pst + i);
+    for (int z = z0; z < zend; ++z) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) c[k] = c[k + 1];
+      c[4] = ldu(u + wrap2(z + 2, d.nz) * pst + i);
+      const double* const up = u + z * pst;
+      const float2 wx = ldw(w + z * pst + i), wy = ldw(w + n + z * pst + i), wz = ldw(w + 2 * n + z * pst + i);
+      const double2 y1 = ldu(up + ym), y2 = ldu(up + yp);
+      double2 y0 = y1, y3 = y2;
+      if (ORDER == 4) {
+        y0 = ldu(up + ymm);
+        y3 = ldu(up + ypp);
       }
-    });
+      const double2 a = ldu(up + xm), b = ldu(up + xp);
+      double xl = 0.0, xr = 0.0;
+      if (W == 1 && ORDER == 4) {
+        xl = __ldg(up + xmm);
+        xr = __ldg(up + xpp);
+      }
+      auto cells = [&](auto f64) {
+        if constexpr (W == 2) {
+          term(vx, f64(wx.x), a.x, a.y, c[2].y, b.x);
+          term(vx, f64(wx.y), a.y, c[2].x, b.x, b.y);
+          term(vy, f64(wy.y), y0.y, y1.y, y2.y, y3.y);
+          term(vz, f64(wz.y), c[0].y, c[1].y, c[3].y, c[4].y);
+        } else {
+          term(vx, f64(wx.x), xl, a.x, b.x, xr);
+        }
+        term(vy, f64(wy.x), y0.x, y1.x, y2.x, y3.x);
+        term(vz, f64(wz.x), c[0].x, c[1].x, c[3].x, c[4].x);
+      };
+      // (one branch for the pair: conversions under a predicate would run for every cell)
+      if (widens(wx.x) && widens(wx.y) && widens(wy.x) && widens(wy.y) && widens(wz.x) && widens(wz.y))
+        cells([](float f) { return widen(f); });
+      else
+        cells([](float f) { return (double)f; });
+    }
+    v = (vx + vy) + vz;
   }
   v = block_sum(v, sh);
-  if (is_thread0()) partials[block_linear_id()] = v;
+  if (is_thread0()) partials[block_linear_id()] = v / (ORDER == 4 ? 12.0 : 2.0);
 }
 
 // z planes of one thread: 16 (four planes of the z window are loaded beside them), fewer
