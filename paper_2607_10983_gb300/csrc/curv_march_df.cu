@@ -420,7 +420,9 @@ __global__ void __launch_bounds__(NT, MINB) k_curv_df_march(Dims d, Fields P, Df
   float2 m = bcast(0.f);
   if (A.m) m = f64_to_df(A.m[0]);
   const DfView V(smf, row, lane);
-  float r2 = 0.f, f2 = 0.f;
+  // compensated: a run may be the whole mesh high, and one FP32 chain of 2 x 256 squares was 5e-6
+  // off (the tiles that this kernel replaced summed 16 per thread)
+  DfAcc r2{0.f, 0.f}, f2{0.f, 0.f};
   issue(z0 - 1, 0);
   fetch(z0);
   cp_wait_all();
@@ -462,10 +464,10 @@ __global__ void __launch_bounds__(NT, MINB) k_curv_df_march(Dims d, Fields P, Df
       const long long i = t * pst + off[k];
       A.r[i] = rv;
       if (A.e1) A.e1[i] = __fmaf_rn(A.omega, __fdiv_rn(__fmul_rn(__fmul_rn(Jc[k], rv), A.h2), Dc[k]), 0.f);
-      r2 += rv * rv;
+      r2.add(__fmul_rn(rv, rv));
       if (A.pf2) {
         const float fv = A.scale_J ? (bc[k].x + bc[k].y) : (bc[k].x + bc[k].y) / Jc[k];
-        f2 += fv * fv;
+        f2.add(__fmul_rn(fv, fv));
       }
     }
     const int q = sc;
@@ -474,11 +476,11 @@ __global__ void __launch_bounds__(NT, MINB) k_curv_df_march(Dims d, Fields P, Df
     sf = q;
   }
   if (A.pr2) {
-    const double s = block_sum_f(r2, shr);
+    const double s = block_sum_acc(r2, shr);
     if (tid == 0) A.pr2[block_linear_id()] = s;
   }
   if (A.pf2) {
-    const double s = block_sum_f(f2, shr);
+    const double s = block_sum_acc(f2, shr);
     if (tid == 0) A.pf2[block_linear_id()] = s;
   }
 }
