@@ -225,6 +225,28 @@ __device__ __forceinline__ double block_sum_acc(const DfAcc& a, double* sh) {
   return block_sum((double)a.s + (double)a.c, sh);
 }
 
+// The same without an FP64 operation per thread: pairs are added across the warp by error-free
+// FP32 sums, then FP64 across warps.
+__device__ __forceinline__ double block_sum_pair(DfAcc a, double* sh) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float s = __shfl_xor_sync(0xffffffffu, a.s, o), c = __shfl_xor_sync(0xffffffffu, a.c, o);
+    a.add(s);
+    a.c += c;
+  }
+  const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
+  const int nt = blockDim.x * blockDim.y * blockDim.z;
+  __syncthreads();
+  if ((tid & 31) == 0) sh[tid >> 5] = (double)a.s + (double)a.c;
+  __syncthreads();
+  double r = 0.0;
+  if (tid < 32) {
+    r = tid < (nt + 31) / 32 ? sh[tid] : 0.0;
+    r = warp_sum(r);
+  }
+  return r;
+}
+
 __device__ __forceinline__ int block_linear_id() {
   return blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
 }

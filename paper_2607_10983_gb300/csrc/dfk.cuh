@@ -42,12 +42,17 @@ __device__ __forceinline__ void st_df2(float2* p, const DF2& v) {
 
 // One tile (x0, y0) and z range [z0, zend) of the fused update and residual; the
 // thread's sums of r'^2, phi' and (F - m)^2 are added to r2, ps, f2 (the caller
-// reduces them).  smf: 3 * TL::PLANE floats of shared memory.  Ends with a barrier.
-template <class TL>
+// reduces them).  flush(r2, f2) is called after every eight planes, for callers whose ranges are
+// long (at most 32 squares in one FP32 chain).  smf: 3 * TL::PLANE floats of shared memory.  Ends
+// with a barrier.
+struct KeepSums {
+  __device__ __forceinline__ void operator()(float&, float&) const {}
+};
+template <class TL, class Flush = KeepSums>
 __device__ __forceinline__ void df_segment(Dims d, const float2* __restrict__ phi_in, const float* __restrict__ e,
                                            const float2* __restrict__ F, const DF2 m, float2* __restrict__ phi_out,
                                            float* __restrict__ r_out, int x0, int y0, int z0, int zend, float* smf,
-                                           float& r2, PAcc& ps, float& f2) {
+                                           float& r2, PAcc& ps, float& f2, Flush flush = Flush()) {
   constexpr int R = TL::R, WXP = TL::WXP, WS = TL::WS, ARR = TL::ARR, PAD = TL::PAD;
   constexpr int PLANE = TL::PLANE;
   const int tid = threadIdx.x;
@@ -143,6 +148,7 @@ __device__ __forceinline__ void df_segment(Dims d, const float2* __restrict__ ph
           f2 = __fmaf_rn(fv.x, fv.x, f2);
           f2 = __fmaf_rn(fv.y, fv.y, f2);
         }
+        if (((zp - z0) & 7) == 7) flush(r2, f2);
       }
       __syncthreads();
     }
