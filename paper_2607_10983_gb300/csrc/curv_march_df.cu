@@ -420,9 +420,17 @@ __global__ void __launch_bounds__(NT, MINB) k_curv_df_march(Dims d, Fields P, Df
   float2 m = bcast(0.f);
   if (A.m) m = f64_to_df(A.m[0]);
   const DfView V(smf, row, lane);
-  // compensated: a run may be the whole mesh high, and one FP32 chain of 2 x 256 squares was 5e-6
-  // off (the tiles that this kernel replaced summed 16 per thread)
-  DfAcc r2{0.f, 0.f}, f2{0.f, 0.f};
+  // with compensation every four planes (8 squares): a run may be the whole mesh high, and one
+  // FP32 chain of 2 x 256 squares was 5e-6 off (the tiles that this kernel replaced summed 16 per
+  // thread).  In shared memory: four more registers across the loop cost 2%.
+  __shared__ DfAcc sums[2][NT];
+  sums[0][tid] = sums[1][tid] = DfAcc{0.f, 0.f};
+  float r2 = 0.f, f2 = 0.f;
+  auto flush = [&]() {
+    sums[0][tid].add(r2);
+    if (A.pf2) sums[1][tid].add(f2);
+    r2 = f2 = 0.f;
+  };
   issue(z0 - 1, 0);
   fetch(z0);
   cp_wait_all();
@@ -464,23 +472,24 @@ __global__ void __launch_bounds__(NT, MINB) k_curv_df_march(Dims d, Fields P, Df
       const long long i = t * pst + off[k];
       A.r[i] = rv;
       if (A.e1) A.e1[i] = __fmaf_rn(A.omega, __fdiv_rn(__fmul_rn(__fmul_rn(Jc[k], rv), A.h2), Dc[k]), 0.f);
-      r2.add(__fmul_rn(rv, rv));
+      r2 = __fmaf_rn(rv, rv, r2);
       if (A.pf2) {
         const float fv = A.scale_J ? (bc[k].x + bc[k].y) : (bc[k].x + bc[k].y) / Jc[k];
-        f2.add(__fmul_rn(fv, fv));
+        f2 = __fmaf_rn(fv, fv, f2);
       }
     }
+    if ((t & 3) == 3 || t + 1 == zend) flush();
     const int q = sc;
     sc = sn;
     sn = sf;
     sf = q;
   }
   if (A.pr2) {
-    const double s = block_sum_acc(r2, shr);
+    const double s = block_sum_pair(sums[0][tid], shr);
     if (tid == 0) A.pr2[block_linear_id()] = s;
   }
   if (A.pf2) {
-    const double s = block_sum_acc(f2, shr);
+    const double s = block_sum_pair(sums[1][tid], shr);
     if (tid == 0) A.pf2[block_linear_id()] = s;
   }
 }
