@@ -110,7 +110,7 @@ gbmg_status curv_cycle(gbmg_ctx* c, bool tr, float* r0, CurvBufs& b) {
   const Level& L0 = c->lv[0];
   double* sc = c->scal;
   TRYS(curv_cycle_step(c, tr, r0, b));
-  TRY(launch_finalize(c->stream, c->partials, curv_df_partials(L0.d, curv_form(c, tr)), sc + S_R2, 1.0));
+  TRY(launch_norm_sum(c->stream, c->partials, curv_df_partials(L0.d, curv_form(c, tr)), sc + S_R2));
   TRY(launch_scalars_to_host(c->stream, c->scal, c->host_scal_dev, 8));
   return GBMG_OK;
 }
@@ -165,8 +165,8 @@ gbmg_status curv_solve_impl(gbmg_ctx* c, const double* src, const double* u_in, 
     c->curv_phi = st.cycles % 2 ? c->phi_df2 : c->phi_df;
     return GBMG_OK;
   }
-  TRY(launch_finalize(c->stream, part, pc, sc + S_R2, 1.0));
-  TRY(launch_finalize(c->stream, part1, pc, sc + S_F2, 1.0));
+  TRY(launch_norm_sum(c->stream, part, pc, sc + S_R2));
+  TRY(launch_norm_sum(c->stream, part1, pc, sc + S_F2));
   double rel = 0.0;
   TRYS(read_rel(c, rel));
   Monitor mon(st, tol, maxv);

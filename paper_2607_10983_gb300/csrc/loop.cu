@@ -114,7 +114,19 @@ __global__ void __launch_bounds__(LT) k_loop_check(const double* __restrict__ pa
   report(L, H);
 }
 
+__global__ void __launch_bounds__(LT) k_norm_sum(const double* __restrict__ p, long long n, double* __restrict__ out) {
+  __shared__ double sh[4];
+  const double s = sum_partials(p, n, sh);
+  if (threadIdx.x == 0) *out = s;
+}
+
 }  // namespace
+
+cudaError_t launch_norm_sum(cudaStream_t st, const double* part, long long n, double* out) {
+  k_norm_sum<<<1, LT, 0, st>>>(part, n, out);
+  note_launch();
+  return cudaGetLastError();
+}
 
 cudaError_t launch_loop_begin(cudaStream_t st, const double* pr2, const double* pf2, long long n, double tol, int maxv,
                               double* r2_out, double* f2_out, LoopState* L, LoopState* H) {

@@ -8,6 +8,9 @@ namespace gbmg {
 // starts the books in L (device) and H (the device address of mapped host memory).
 cudaError_t launch_loop_begin(cudaStream_t st, const double* pr2, const double* pf2, long long n, double tol, int maxv,
                               double* r2_out, double* f2_out, LoopState* L, LoopState* H);
+// The sum of n partials in the order of the loop's checks, for the solves that the host drives:
+// their histories have the same bits.
+cudaError_t launch_norm_sum(cudaStream_t st, const double* part, long long n, double* out);
 cudaError_t launch_loop_gate(cudaStream_t st, const LoopState* L, cudaGraphConditionalHandle w);
 cudaError_t launch_loop_check(cudaStream_t st, const double* part, long long n, double* r2_out, LoopState* L,
                               LoopState* H, cudaGraphConditionalHandle w, cudaGraphConditionalHandle f, int second);

@@ -322,10 +322,10 @@ gbmg_status solve_fp64(gbmg_ctx* c, const double* F, double* phi, double tol, in
     return loop_result(c, c->loop_kernels[0], st);
   }
   TRY(launch_sum<double>(c->stream, n, f0, nullptr, part));
-  TRY(launch_finalize(c->stream, part, pr, sc + S_F2, 1.0));
+  TRY(launch_norm_sum(c->stream, part, pr, sc + S_F2));
   auto resnorm = [&]() -> gbmg_status {
     TRYS(residual(part));
-    TRY(launch_finalize(c->stream, part, pc, sc + S_R2, 1.0));
+    TRY(launch_norm_sum(c->stream, part, pc, sc + S_R2));
     return GBMG_OK;
   };
   TRYS(resnorm());
@@ -367,7 +367,7 @@ gbmg_status fused_cycle_step(gbmg_ctx* c, const float2* phi_cur, float2* phi_nxt
 // stream is synchronised).
 gbmg_status fused_cycle(gbmg_ctx* c, const float2* phi_cur, float2* phi_nxt, float* r0, float* r_nxt) {
   TRYS(fused_cycle_step(c, phi_cur, phi_nxt, r0, r_nxt));
-  TRY(launch_finalize(c->stream, c->partials, df_update_residual_partials(c->lv[0].d), c->scal + S_R2, 1.0));
+  TRY(launch_norm_sum(c->stream, c->partials, df_update_residual_partials(c->lv[0].d), c->scal + S_R2));
   TRY(launch_scalars_to_host(c->stream, c->scal, c->host_scal_dev, 8));
   return GBMG_OK;
 }
@@ -423,8 +423,8 @@ gbmg_status solve_mixed(gbmg_ctx* c, const double* F, const double* phi, double*
       TRY(launch_df_to_f64(c->stream, n, c->phi_df, sc + S_MEAN_PHI, phi_out, c->phi_df2, &c->loop_dev->cycles));
       return loop_result(c, c->loop_kernels[0], st);
     }
-    TRY(launch_finalize(c->stream, part, pu, sc + S_R2, 1.0));
-    TRY(launch_finalize(c->stream, part1, pu, sc + S_F2, 1.0));
+    TRY(launch_norm_sum(c->stream, part, pu, sc + S_R2));
+    TRY(launch_norm_sum(c->stream, part1, pu, sc + S_F2));
   } else {
     TRY(launch_df_residual(c->stream, L0.d, c->F_df, sc + S_MEAN_F, c->phi_df, r0, part, part1));
     TRY(launch_finalize(c->stream, part, pc, sc + S_R2, 1.0));
