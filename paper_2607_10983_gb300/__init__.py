@@ -417,7 +417,8 @@ class Solver:
 
     # -- measurement
     def set_cycle_graphs(self, enable: bool):
-        """Run each V-cycle as one CUDA graph launch (default) or launch every kernel eagerly."""
+        """Run a solve's V-cycles as one CUDA graph that loops on the device (default) or launch every
+        kernel from the host."""
         _check(lib().mg_set_cycle_graphs(self._c(), 1 if enable else 0))
 
     def profile_begin(self, families):
@@ -510,7 +511,8 @@ class Solver:
 
 
 class Batch:
-    """Independent flat solves of uneven sizes in one persistent launch (mg_batch_*)."""
+    """Independent flat solves of uneven sizes (mg_batch_*): one persistent launch, or with
+    use_graph a graph of phase kernels."""
 
     def __init__(self, shapes, degree: int = 3, levels: int = 0, coarse_store: str = "fp32"):
         self.solvers = [Solver(s, levels=levels, degree=degree, prec="mixed", fused=False, coarse_store=coarse_store)

@@ -18,7 +18,7 @@
 // max_vcycles is reached.  Per-problem completion times come from %globaltimer.
 //
 // With mg_batch_use_graph the phases run as kernels of a graph instead where every level is
-// fused or in a bottom cycle (batch_graph.cu): 48 problems 13.0 ms launched here, 8.2 there.
+// fused or in a bottom cycle (batch_graph.cu): 48 problems 13.6 ms launched here, 7.9 there.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -94,6 +94,29 @@ __device__ __forceinline__ void phase(const BDesc& B, int l, Want want, Op op) {
     const long long s1 = s0 + B.chunk[l] < n ? s0 + B.chunk[l] : n;
     for (long long i = s0 + threadIdx.x; i < s1; i += blockDim.x) op(P, l, i);
   }
+}
+
+// Level-0 phase with a per-chunk partial sum of the float returned by op.
+template <typename Op>
+__device__ __forceinline__ void phase0_sum(const BDesc& B, double* part, double* sh, bool all, Op op) {
+  for (int c = blockIdx.x; c < B.nchunk[0]; c += gridDim.x) {
+    const int pi = B.cprob[0][c];
+    if (!all && B.status[pi] != ST_ACTIVE) continue;
+    const BProb& P = B.p[pi];
+    const long long s0 = B.cstart[0][c];
+    const long long n = ncell(P.d[0]);
+    const long long s1 = s0 + B.chunk[0] < n ? s0 + B.chunk[0] : n;
+    DfAcc acc{0.f, 0.f};
+    for (long long i = s0 + threadIdx.x; i < s1; i += blockDim.x) op(P, i, acc);
+    const double b = block_sum_acc(acc, sh);
+    if (threadIdx.x == 0) part[c] = b;
+  }
+}
+
+__device__ __forceinline__ double chunk_total(const BDesc& B, const BProb& P, const double* part) {
+  double s = 0.0;
+  for (int k = 0; k < P.nch; ++k) s += part[P.c0 + k];
+  return s;
 }
 
 // Fused phases: the (problem, tile, plane) list of level l, split evenly over the

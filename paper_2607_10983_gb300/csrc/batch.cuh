@@ -1,5 +1,5 @@
-// Descriptors of the batched solves and the device helpers that the persistent kernel
-// (batch.cu) and the kernels of the phase graph (batch_graph.cu) share.
+// What the persistent kernel of the batched solves (batch.cu) and the kernels of their phase
+// graph (batch_graph.cu) share: descriptors and a few device helpers.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -87,29 +87,6 @@ __device__ __forceinline__ unsigned long long globaltimer() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
   return t;
-}
-
-// Level-0 phase with a per-chunk partial sum of the float returned by op.
-template <typename Op>
-__device__ __forceinline__ void phase0_sum(const BDesc& B, double* part, double* sh, bool all, Op op) {
-  for (int c = blockIdx.x; c < B.nchunk[0]; c += gridDim.x) {
-    const int pi = B.cprob[0][c];
-    if (!all && B.status[pi] != ST_ACTIVE) continue;
-    const BProb& P = B.p[pi];
-    const long long s0 = B.cstart[0][c];
-    const long long n = ncell(P.d[0]);
-    const long long s1 = s0 + B.chunk[0] < n ? s0 + B.chunk[0] : n;
-    DfAcc acc{0.f, 0.f};
-    for (long long i = s0 + threadIdx.x; i < s1; i += blockDim.x) op(P, i, acc);
-    const double b = block_sum_acc(acc, sh);
-    if (threadIdx.x == 0) part[c] = b;
-  }
-}
-
-__device__ __forceinline__ double chunk_total(const BDesc& B, const BProb& P, const double* part) {
-  double s = 0.0;
-  for (int k = 0; k < P.nch; ++k) s += part[P.c0 + k];
-  return s;
 }
 
 // level l of problem P runs the fused legs

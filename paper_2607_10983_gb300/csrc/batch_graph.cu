@@ -4,8 +4,10 @@
 // The persistent kernel holds every phase under one register limit at 12 warps per SM, so
 // its phases ran 1.5 to 2 times as long as the kernels of single solves: 14.3 ms for 48
 // problems of 64^3, 96^3 and 128^3, seven cycles (finest level per cycle: down 372, up 532,
-// update 595 us; here 8.4 ms, the update 323 us, all down legs together 295 and all up legs 387).  As kernels of their own the legs have the
-// single solves' tiles and registers, the double-float step two CTAs per SM, and the bottom
+// update 595 us; here 7.9 ms, the update 323 us, all down legs together 295 and all up legs 387).
+// As kernels of their own the legs have the single solves' tiles and register limits (beside the
+// batch's descriptors the down legs spill 16 bytes at degree 3 and 12 at degree 4, the up leg 4 at
+// degree 4; those of single solves none), the double-float step has two CTAs per SM, and the bottom
 // cycle 1024 threads; a launch boundary costs about what the grid barrier did.  Each value
 // sees the same operations as in the persistent kernel (the chunks of the means and their
 // summation order too), so both give the same iterates bit for bit; the residual norms are
