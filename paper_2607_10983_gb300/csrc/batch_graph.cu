@@ -4,7 +4,7 @@
 // The persistent kernel holds every phase under one register limit at 12 warps per SM, so
 // its phases ran 1.5 to 2 times as long as the kernels of single solves: 14.3 ms for 48
 // problems of 64^3, 96^3 and 128^3, seven cycles (finest level per cycle: down 372, up 532,
-// update 595 us; here 7.9 ms, the update 323 us, all down legs together 295 and all up legs 387).
+// update 595 us; here 7.9 ms, the update 324 us, all down legs together 269 and all up legs 340).
 // As kernels of their own the legs have the single solves' tiles and register limits (beside the
 // batch's descriptors the down legs spill 16 bytes at degree 3 and 12 at degree 4, the up leg 4 at
 // degree 4; those of single solves none), the double-float step has two CTAs per SM, and the bottom
@@ -316,7 +316,7 @@ gbmg_status PhaseGraph::init(const std::vector<gbmg_ctx*>& ctx, const BProb* pro
       long long* const u = o + (size_t)D.maxL * (count + 1);
       u[i + 1] = u[i] + nu;
     }
-  // planes of an update item: 32 (for 48 problems 323 us per cycle; 16 and 48 329, 8 and 128
+  // planes of an update item: 32 (for 48 problems 324 us per cycle; 16 and 48 329, 8 and 128
   // 363), fewer where that leaves less than two items for a CTA's place (two on an SM)
   for (t.fz = 32;; t.fz /= 2) {
     for (int i = 0; i < count; ++i) {

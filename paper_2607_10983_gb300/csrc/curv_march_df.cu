@@ -494,9 +494,10 @@ __global__ void __launch_bounds__(NT, MINB) k_curv_df_march(Dims d, Fields P, Df
   }
 }
 
-// CTAs (of 256 threads) per SM, measured at 256^3 with the update (us; 1, 2, 3 CTAs):
+// CTAs (of 256 threads) per SM, measured at 256^3 with the update and one FP32 chain for the norm
+// (us; 1, 2, 3 CTAs):
 //   M 474, 399, 607 (spills)   M^T 498, 657 (spills), -   S 438, 373, 553 (spills)
-// against 354 / 478 / 400 for the residual alone in the one-cell tiles, the update's 50 and
+// (with the norm's compensated sums M 389, M^T 509, S 364) against 354 / 478 / 400 for the residual alone in the one-cell tiles, the update's 50 and
 // the first sweep's 82 of their own.
 constexpr int kCtas[3] = {2, 1, 2};
 template <class OP, int MINB>

@@ -14,7 +14,8 @@ namespace {
 
 // FP64 runs at under 2 operations per clock on an SM, so the sums take four warps and a
 // tree of theirs, not a block of 1024 threads of which most add zeros (5.9 -> 3.1 us for the
-// 128 partials of 64^3 with the host copy left to the last check).
+// 128 partials of 64^3 alone, with the host copy left to the last check; 4.2 in that solve, up to
+// 6.4 with the thousands of larger meshes).
 constexpr int LT = 128;
 
 // valid in every thread
