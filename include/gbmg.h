@@ -58,6 +58,9 @@ typedef enum { GBMG_FP64 = 0, GBMG_MIXED = 1 } gbmg_prec;
 typedef enum { GBMG_SMOOTH_CHEBYSHEV = 0, GBMG_SMOOTH_JACOBI = 1 } gbmg_smoother;
 typedef enum { GBMG_F32 = 0, GBMG_F64 = 1 } gbmg_dtype;
 
+/* Arguments of mg_set_cycle_graphs and mg_batch_use_graph for tests. */
+enum { GBMG_TEST_REFUSE = 0x7e5701, GBMG_TEST_REFUSE_INSTANTIATE = 0x7e5702 };
+
 /* Solver options.  gbmg_default_opts fills the paper's defaults:
  * Chebyshev degree 3 on [2/alpha, 2] with alpha = 8 (Sec. 2.3, Eq. flat_chebyshev),
  * Jacobi omega = 2/3 with nu1 = nu2 = 2 (Sec. 2.3 Eq. flat_jacobi, Sec. 4.3.3),
@@ -131,9 +134,10 @@ gbmg_status mg_set_stream(gbmg_ctx* ctx, void* cuda_stream);
  * orientation) and launched once per solve, and the host waits once.  While kernel families
  * are timed (mg_profile_begin), each cycle of a mixed solve is a graph launch of its own
  * with event nodes, and the host checks convergence after every cycle.  Results are the
- * same bits either way.  enable = 0 launches every kernel of every cycle from the host;
- * enable = 2 (testing) refuses the context what a driver or a partition of a GPU may refuse:
- * loops in graphs (leaving a graph launch per cycle), cooperative grids and clusters of 16. */
+ * same bits either way.  enable = 0 launches every kernel of every cycle from the host, other
+ * values switch the graphs on.  GBMG_TEST_REFUSE (testing) also refuses the context what a driver
+ * or a partition of a GPU may refuse: loops in graphs (leaving a graph launch per cycle),
+ * cooperative grids and clusters of 16. */
 gbmg_status mg_set_cycle_graphs(gbmg_ctx* ctx, int enable);
 
 /* Curvilinear contexts only: set the deformation potential psi (nx*ny*nz doubles,
@@ -303,9 +307,9 @@ gbmg_status mg_batch_get_tiles(const gbmg_batch* batch, int* tile_cells, int nle
  * sizes are unchanged; ordered after earlier and before later work on the batch's stream).
  * Where every problem has even nx, a bottom cycle (degrees 1 to 4) and no level above it with
  * a side below 16, the graph runs the phases as kernels of their own in a loop on the device
- * (of the grid and tile sizes it reads the level-0 tiles), otherwise the persistent kernel.  on = 2 or 3 (testing) lets the
- * construction or the instantiation of the phase graph fail, which leaves the batch on the
- * persistent kernel.  Off by default. */
+ * (of the grid and tile sizes it reads the level-0 tiles), otherwise the persistent kernel.  GBMG_TEST_REFUSE and
+ * GBMG_TEST_REFUSE_INSTANTIATE (testing) let the construction or the instantiation of the phase
+ * graph fail, which leaves the batch on the persistent kernel.  Off by default. */
 gbmg_status mg_batch_use_graph(gbmg_batch* batch, int on);
 /* Number of levels of the deepest problem (length of the tile-size array). */
 int mg_batch_num_levels(const gbmg_batch* batch);

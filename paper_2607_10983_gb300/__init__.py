@@ -24,6 +24,7 @@ F32, F64 = 0, 1
 OP_FLAT7, OP_CURV19 = 0, 1
 FP64, MIXED = 0, 1
 CHEBYSHEV, JACOBI = 0, 1
+TEST_REFUSE, TEST_REFUSE_INSTANTIATE = 0x7E5701, 0x7E5702  # (of the graph switches, for tests)
 
 STATUS = {0: "ok", 1: "invalid argument", 2: "CUDA error", 3: "out of memory", 4: "not converged",
           5: "non-finite residual", 6: "diverged", 7: "invalid state"}

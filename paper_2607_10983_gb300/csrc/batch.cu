@@ -534,7 +534,7 @@ struct gbmg_batch {
   // reads of the schedule (the phases: the level-0 tile size; the persistent kernel: the grid
   // and every tile size)
   bool use_graph = false;
-  int refuse = 0;   // testing: building (2) or instantiating (3) the phase graph fails
+  int refuse = 0;   // testing (GBMG_TEST_*): building or instantiating the phase graph fails
   cudaStream_t gstream = nullptr;
   cudaEvent_t gev[2] = {nullptr, nullptr};
   cudaGraphExec_t gexec = nullptr;
@@ -965,8 +965,8 @@ extern "C" gbmg_status mg_batch_solve(gbmg_batch* b, const double* const* src_de
       // nodes or with no memory left for them, leaves the batch on the persistent kernel)
       if (b->phases.usable) {
         gbmg_status ps = b->phases.build(b->gstream, D, &graph, [&]() { return copy_in(b->gstream); },
-                                         [&]() { return copy_out(b->gstream); }, b->refuse == 2);
-        if (ps == GBMG_OK && (b->refuse == 3 || cudaGraphInstantiate(&b->gexec, graph, 0) != cudaSuccess))
+                                         [&]() { return copy_out(b->gstream); }, b->refuse == GBMG_TEST_REFUSE);
+        if (ps == GBMG_OK && (b->refuse == GBMG_TEST_REFUSE_INSTANTIATE || cudaGraphInstantiate(&b->gexec, graph, 0) != cudaSuccess))
           ps = GBMG_ERR_CUDA;
         if (graph) cudaGraphDestroy(graph);
         graph = nullptr;

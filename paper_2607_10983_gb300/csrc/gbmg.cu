@@ -299,7 +299,7 @@ extern "C" gbmg_status mg_set_cycle_graphs(gbmg_ctx* ctx, int enable) {
   if (e != cudaSuccess) return cuda_fail(e, "mg_set_cycle_graphs");
   ctx->cyc_off = enable == 0;
   if (enable) ctx->loop_off = false;
-  ctx->refuse = enable == 2;
+  ctx->refuse = enable == GBMG_TEST_REFUSE;
   ctx->graph_mask = -1;  // drop the graphs captured so far
   sync_graph_mask(ctx);
   return GBMG_OK;

@@ -16,7 +16,7 @@ def test_bottom_without_a_cluster(gb, shape, degree):
         s = gb.Solver(shape, prec="fp64", degree=degree)
         s.set_cycle_graphs(False)
         if refuse:
-            gb._check(gb.lib().mg_set_cycle_graphs(s._c(), 2))
+            gb._check(gb.lib().mg_set_cycle_graphs(s._c(), gb.TEST_REFUSE))
         n = gb.launch_count()
         e = s.vcycle(F)
         n = gb.launch_count() - n

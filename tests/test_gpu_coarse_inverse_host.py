@@ -15,7 +15,7 @@ torch = pytest.importorskip("torch")
 def test_host_inverse_has_the_kernels_bits(gb, shape, levels, sym):
     psi = torch.from_numpy(smoothed_grf(shape, 100, 1.0, 0.4)).cuda()
     gpu, host = (gb.Solver(shape, op="curv", levels=levels, curv_sym=sym) for _ in range(2))
-    gb._check(gb.lib().mg_set_cycle_graphs(host._c(), 2))
+    gb._check(gb.lib().mg_set_cycle_graphs(host._c(), gb.TEST_REFUSE))
     F = torch.randn(shape, generator=torch.Generator(device="cuda").manual_seed(101), device="cuda", dtype=torch.float64)
     r = torch.randn(gpu.level_shape(gpu.levels - 1), generator=torch.Generator(device="cuda").manual_seed(102),
                     device="cuda", dtype=torch.float64)

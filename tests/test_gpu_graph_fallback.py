@@ -16,7 +16,7 @@ def test_flat_solve_without_its_loop(gb, prec, krylov):
     F = torch.from_numpy(grf(SHAPE, 320)).cuda()
     eager, refused = (gb.Solver(SHAPE, prec=prec, krylov=krylov) for _ in range(2))
     eager.set_cycle_graphs(False)
-    gb._check(gb.lib().mg_set_cycle_graphs(refused._c(), 2))
+    gb._check(gb.lib().mg_set_cycle_graphs(refused._c(), gb.TEST_REFUSE))
     for tol in (1e-9, 1e-4):
         pe, se = eager.solve(F, tol=tol)
         pr, sr = refused.solve(F, tol=tol)
@@ -35,7 +35,7 @@ def test_curvilinear_solve_without_its_loop(gb, sym):
     bar = torch.from_numpy(np.random.default_rng(323).standard_normal(SHAPE)).cuda()
     eager, refused = (gb.Solver(SHAPE, op="curv", curv_sym=sym) for _ in range(2))
     eager.set_cycle_graphs(False)
-    gb._check(gb.lib().mg_set_cycle_graphs(refused._c(), 2))
+    gb._check(gb.lib().mg_set_cycle_graphs(refused._c(), gb.TEST_REFUSE))
     for tol in (1e-7, 1e-4):
         got = []
         for s in (eager, refused):
@@ -46,14 +46,14 @@ def test_curvilinear_solve_without_its_loop(gb, sym):
         assert all(torch.equal(a, b) for a, b in zip(got[0][:3], got[1][:3]))
 
 
-@pytest.mark.parametrize("refusal", [2, 3])   # of its construction, of its instantiation
+@pytest.mark.parametrize("refusal", ["TEST_REFUSE", "TEST_REFUSE_INSTANTIATE"])
 @pytest.mark.parametrize("degree", [1, 3])
 def test_batch_without_its_phase_graph(gb, degree, refusal):
     shapes = [(32, 32, 32), (64, 48, 64)]
     F = [torch.from_numpy(grf(s, 324 + i)).cuda() for i, s in enumerate(shapes)]
     batch = gb.Batch(shapes, degree=degree)
     got = []
-    for mode in (0, refusal, refusal):
+    for mode in (0, getattr(gb, refusal), getattr(gb, refusal)):
         gb._check(gb.lib().mg_batch_use_graph(batch._b, mode))
         phi = [torch.zeros_like(f) for f in F]
         stats, _ = batch.solve(F, phi, tol=1e-8)
