@@ -18,7 +18,7 @@ def test_norm_of_a_long_column(gb, sym):
     s = gb.Solver(shape, op="curv", curv_sym=sym)
     _, st = s.solve(f * sign, (r - f) / 12.0 * sign, tol=0.0, max_vcycles=0, psi=torch.zeros(shape, dtype=torch.float64,
                                                                                             device="cuda"))
-    # the two squares and the residual, rounded to FP32 once each: 2^-25 (2 x 1/2 + 1), and the sums
-    # far below; 2^-22 leaves room for the double-float residual
+    # chains of eight squares, each addition half an ulp of at most its partial sum: 4 x 2^-24 of
+    # either sum at worst, half of it on each root, together 2^-22
     assert abs(st.rel_res0 / (r / f) - 1.0) <= 2.0 ** -22
     s.close()
